@@ -114,10 +114,11 @@ typedef struct {
 
 enum {
   REWL_RESOLVER_AUTO = 0,       /* per batch: the cheapest of the three for the last batch's events */
-  REWL_RESOLVER_SCAN = 1,       /* one 64-bit warp prefix scan of the energy increments, one ballot
-                                   round per event (bin change, correction) */
-  REWL_RESOLVER_BLOCKS = 2,     /* branch-free blocks of 8 moves; events leave the block */
-  REWL_RESOLVER_SEQUENTIAL = 3  /* one move at a time */
+  REWL_RESOLVER_SCAN = 1,       /* runs of moves that stay in the bin, from one warp prefix sum of the
+                                   energy increments; one round per move that leaves the bin */
+  REWL_RESOLVER_BLOCKS = 2,     /* blocks of moves up to the next accepted one, one round each, steps to a
+                                   neighbouring bin decided by two pass bits per move */
+  REWL_RESOLVER_SEQUENTIAL = 3  /* one accepted move after the other, every move's target bin looked up */
 };
 
 typedef struct {
@@ -159,7 +160,7 @@ typedef struct {
                                   memory, moves sharing a conflict-table entry count too (the table
                                   has an entry per site up to 8192 sites) */
   int64_t batches_scan;        /* production, warp-specialised walker: batches of 32 moves resolved */
-  int64_t batches_blocks;      /*   by the warp scan, by 8-move blocks and one move at a time */
+  int64_t batches_blocks;      /*   by the warp scan, by blocks and one accepted move at a time */
   int64_t batches_sequential;  /*   (all 0 for the other walkers and in trajectory mode) */
 } rewl_counters;
 

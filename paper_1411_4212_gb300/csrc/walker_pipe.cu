@@ -9,12 +9,11 @@
 //     resolved while batch b+1 reads the lattice) and the earlier moves of batch b+1 that sit on the
 //     same site or a neighbouring one;
 //   resolver: a move whose mask meets a move accepted since the lattice was read is corrected
-//     exactly (production: from the move records; trajectory: re-evaluated on the current lattice);
+//     exactly (production: from the move batches; trajectory: re-evaluated on the current lattice);
 //     then accept with min[1, g(E)/g(E')] (reject outside the window) and add ln f to ln g and 1 to
 //     H at the resulting state.
-// The owner table may alias sites (hashed): an alias names a move that cannot change the field, so
-// its correction changes nothing, and the production walker over a global lattice drops it before
-// it becomes an event.  Two record buffers alternate; named barriers READY(b mod 2) and DONE(b mod 2)
+// The owner table may alias sites (hashed): an alias names a move that cannot change the field; the
+// production producer sorts such bits out by the distance of the sites.  Two record buffers alternate; named barriers READY(b mod 2) and DONE(b mod 2)
 // order the hand-over, so the producer reads the lattice only after every move of batch b-1 has been
 // written.
 #include <cstring>
@@ -62,23 +61,27 @@ __device__ __forceinline__ void named_arrive(int id) {
   asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(kPairThreads) : "memory");
 }
 
-template <bool kTraj>
-struct alignas(16) Rec;
-template <>
-struct alignas(16) Rec<false> {
-  long long dq;          // energy increment, 2^-32 bins (a 2^-24-bin integer shifted left by 8)
-  int lu;                // ln u, 2^-20 units
-  uint32_t cprev;        // batch b-1 moves touching this move's neighbourhood
-  uint32_t ccur;         // earlier moves of this batch touching it
-  int site;
-  float nx, ny, nz;      // proposed spin
-  float ox, oy, oz;      // spin at the site before the move (snapshot, corrected by the resolver)
-  float hx, hy, hz;      // local field (snapshot, corrected by the resolver)
-  float dsx, dsy, dsz;   // new - old spin: the move's change to the lattice if accepted
-  float cu, cv;          // octahedral code of the proposed spin (what the lattice stores)
+// Production: one batch of 32 trial moves as the producer hands it over, one entry per move.  Every
+// section is an array of 16-byte words, so the resolver's reads (lane = move, or any other move of the
+// batch) are conflict-free 16-byte loads.  A move touches another when it sits on the other's site or on
+// one of its neighbours; the masks hold the moves that touch this one, by the shell they sit on.
+struct alignas(16) MoveBatch {
+  int4 head[32];         // energy increment (2^-24 bins) | ln u (2^-20 units) | moves of batch b-1 touching
+                         // this one | earlier moves of this batch touching it (both as they are counted)
+  int4 place[32];        // site | octahedral code (u, v) of the proposed spin, what the lattice stores
+  float4 n[32];          // proposed spin | earlier moves of this batch on this site
+  float4 h[32];          // local field (snapshot) | moves of batch b-1 on this site (bits reversed: move j
+                         // is bit 31 - j, so that count-leading-zeros walks them in order)
+  float4 ds[32];         // new - old spin: the move's change to the lattice if accepted (kept current by
+                         // the resolver) | half-unit coordinates X | Y << 10 | Z << 20
+  int4 cur[32];          // earlier moves of this batch on a neighbour, by shell
+  int4 prev[32];         // moves of batch b-1 on a neighbour, by shell (bits reversed)
+  int4 all;              // moves that touch a later one | moves on a later one's site | moves whose
+                         // increment is a bin or more (count)
 };
-template <>
-struct alignas(16) Rec<true> {
+
+// Trajectory: one move.
+struct alignas(16) TrajRec {
   double dE;
   double u;
   uint32_t cprev, ccur;
@@ -86,13 +89,18 @@ struct alignas(16) Rec<true> {
   double nx, ny, nz, pad2;
 };
 
+// Bytes of the two move batches in flight.
+__host__ __device__ constexpr size_t batch_bytes(bool traj) {
+  return traj ? 64 * sizeof(TrajRec) : 2 * sizeof(MoveBatch);
+}
+
 // Local field of (X, Y, Z) by one lane over all slots in canonical order, with the owner-table
-// words of the site's neighbours OR-ed into own0 / own1 (kOwn).
-template <bool kTraj, int NSH, bool kOwn = true, class Lat>
+// words of the site's neighbours OR-ed into own[shell].
+template <bool kTraj, int NSH, class Lat>
 __device__ __forceinline__ void field_one_lane(const Lat& lat, int X, int Y, int Z, int L, const typename Mode<kTraj>::Real (&Jsh)[4],
                                                typename Mode<kTraj>::Real& hx, typename Mode<kTraj>::Real& hy,
                                                typename Mode<kTraj>::Real& hz, const uint2* own, uint32_t omask,
-                                               uint32_t& own0, uint32_t& own1) {
+                                               uint2 (&touch)[4]) {
   using Real = typename Mode<kTraj>::Real;
   constexpr ShellTable T = make_shells(NSH);
   const int twoL = 2 * L, LL = L * L;
@@ -135,11 +143,9 @@ __device__ __forceinline__ void field_one_lane(const Lat& lat, int X, int Y, int
       ty[T.sh[j]] += vy;
       tz[T.sh[j]] += vz;
     }
-    if constexpr (kOwn) {
-      const uint2 o = own[n & omask];
-      own0 |= o.x;
-      own1 |= o.y;
-    }
+    const uint2 o = own[n & omask];
+    touch[T.sh[j]].x |= o.x;
+    touch[T.sh[j]].y |= o.y;
   }
   if constexpr (!kTraj) {
 #pragma unroll
@@ -180,8 +186,8 @@ __device__ __forceinline__ void pipe_walk_slot(const WalkerArgs& a, const int sl
   const int rep = a.st.perm[slot];
   const uint32_t omask = (uint32_t)a.own_mask;
 
-  // shared layout: ln g | H | offsets | J per slot | records[2][32] | packed records[2][32] | owner
-  // table | lattice (in shared memory only); every section starts on a 16-byte boundary
+  // shared layout: ln g | H | offsets | J per slot | move batches [2] | owner table | lattice (in shared
+  // memory only); every section starts on a 16-byte boundary
   unsigned char* p = smem_raw;
   Lng* lng_s = reinterpret_cast<Lng*>(p);
   p += align16(sizeof(Lng) * (size_t)W);
@@ -191,10 +197,9 @@ __device__ __forceinline__ void pipe_walk_slot(const WalkerArgs& a, const int sl
   p += 4 * kMaxSlotsPerSite;
   Real* J_s = reinterpret_cast<Real*>(p);
   p += sizeof(Real) * kMaxSlotsPerSite;
-  Rec<kTraj>* rec = reinterpret_cast<Rec<kTraj>*>(p);
-  p += sizeof(Rec<kTraj>) * 64;
-  int4* pk = reinterpret_cast<int4*>(p);          // production: {dq lo, dq hi, ccur, ln u} per move
-  p += sizeof(int4) * 64;
+  TrajRec* rec = reinterpret_cast<TrajRec*>(p);            // trajectory: [2][32]
+  MoveBatch* mb = reinterpret_cast<MoveBatch*>(p);         // production: [2]
+  p += batch_bytes(kTraj);
   uint2* own = reinterpret_cast<uint2*>(p);
   p += sizeof(uint2) * ((size_t)omask + 1);
   Real* spin_s = reinterpret_cast<Real*>(p);
@@ -233,6 +238,7 @@ __device__ __forceinline__ void pipe_walk_slot(const WalkerArgs& a, const int sl
     for (int s2 = 0; s2 < 4; ++s2) Jsh[s2] = kTraj ? (Real)a.geo.Jsh_d[s2] : (Real)a.geo.Jsh_f[s2];
     int site_prev = 0;
     bool valid_prev = false;
+    const bool aliased = (long long)omask + 1 < (long long)N;   // several sites share an owner entry
     for (int b = 0; b < nb; ++b) {
       const int cur = b & 1;
       const bool valid = (long long)b * 32 + lane < moves;
@@ -271,50 +277,89 @@ __device__ __forceinline__ void pipe_walk_slot(const WalkerArgs& a, const int sl
       uint32_t* own32 = reinterpret_cast<uint32_t*>(own);
       if (valid) atomicOr(own32 + 2 * (site & omask) + cur, 1u << lane);
       __syncwarp();
-      uint32_t o0 = 0, o1 = 0;
+      uint2 touch[4] = {};
       Real hx, hy, hz;
       // the draws and the owner-table insert above do not touch the lattice, so they overlap the
       // resolver's publication of batch b-2; the lattice holds every batch up to b-2 after DONE
       if (b >= 2) named_sync(kBarDone + (b & 1));
-      field_one_lane<kTraj, NSH>(lat, X, Y, Z, L, Jsh, hx, hy, hz, own, omask, o0, o1);
+      field_one_lane<kTraj, NSH>(lat, X, Y, Z, L, Jsh, hx, hy, hz, own, omask, touch);
       const uint2 oself = own[site & omask];
-      o0 |= oself.x;
-      o1 |= oself.y;
-      const uint32_t ocur = cur ? o1 : o0, oprev = cur ? o0 : o1;
       Real ox, oy, oz;
       lat.get(site, ox, oy, oz);
-      Rec<kTraj>& r = rec[cur * 32 + lane];
+      // moves on this site and on the neighbours of each shell: earlier ones of this batch, and those of
+      // batch b-1
+      const uint32_t below = (1u << lane) - 1u, any_prev = b > 0 ? 0xffffffffu : 0u;
+      uint32_t scur = (cur ? oself.y : oself.x) & below, sprev = (cur ? oself.x : oself.y) & any_prev;
+      uint32_t tcur[4], tprev[4], ccur = scur, cprev = sprev;
+#pragma unroll
+      for (int s2 = 0; s2 < 4; ++s2) {
+        tcur[s2] = (cur ? touch[s2].y : touch[s2].x) & below;
+        tprev[s2] = (cur ? touch[s2].x : touch[s2].y) & any_prev;
+        ccur |= tcur[s2];
+        cprev |= tprev[s2];
+      }
       if constexpr (kTraj) {
+        TrajRec& r = rec[cur * 32 + lane];
         const double dx = __dsub_rn(nx, ox), dy = __dsub_rn(ny, oy), dz = __dsub_rn(nz, oz);
         r.dE = -__dadd_rn(__dadd_rn(__dmul_rn(dx, hx), __dmul_rn(dy, hy)), __dmul_rn(dz, hz));
         r.u = u;
+        r.cprev = cprev;
+        r.ccur = ccur;
+        r.site = site;
+        r.nx = nx;
+        r.ny = ny;
+        r.nz = nz;
       } else {
-        const float dx = nx - ox, dy = ny - oy, dz = nz - oz;
+        MoveBatch& m = mb[cur];
+        // (rounded subtractions: a plain one could fuse with the product that decoded the old spin)
+        const float dx = __fsub_rn(nx, ox), dy = __fsub_rn(ny, oy), dz = __fsub_rn(nz, oz);
         const float dE = -fmaf(dz, hz, fmaf(dy, hy, dx * hx));
-        r.dq = (long long)dq24_of(dE, a.win) << 8;
-        r.lu = lu;
-        r.ox = ox;
-        r.oy = oy;
-        r.oz = oz;
-        r.hx = hx;
-        r.hy = hy;
-        r.hz = hz;
-        r.dsx = dx;
-        r.dsy = dy;
-        r.dsz = dz;
-        r.cu = code.x;
-        r.cv = code.y;
+        const int dq = dq24_of(dE, a.win);
+        m.ds[lane] = make_float4(dx, dy, dz, __int_as_float(X | (Y << 10) | (Z << 20)));
+        if (aliased) {
+          // An owner table smaller than the lattice is hashed: a bit may name a move whose site is neither
+          // this move's site nor one of its neighbours, or name a shell that it does not sit on.  Sort the
+          // bits by the distance of the sites.  With the lattice in global memory only real conflicts
+          // count.  (At bcc L = 32 with 2048 entries, 92 % of the flagged moves were aliases.)
+          __syncwarp();
+          auto sort_bits = [&](const MoveBatch& other, uint32_t bits, uint32_t& same, uint32_t (&sh)[4]) {
+            same = sh[0] = sh[1] = sh[2] = sh[3] = 0u;
+            for (; bits; bits &= bits - 1u) {
+              const int j = __ffs(bits) - 1;
+              const uint32_t q = __float_as_uint(other.ds[j].w), bit = 1u << j;
+              // every offset component of a neighbour is below L half-units, so the wrapped displacement
+              // is the offset; squared distances 3, 4, 8, 11 are the shells 1..4
+              int ex = abs((int)(q & 1023u) - X), ey = abs((int)((q >> 10) & 1023u) - Y), ez = abs((int)(q >> 20) - Z);
+              ex = min(ex, 2 * L - ex);
+              ey = min(ey, 2 * L - ey);
+              ez = min(ez, 2 * L - ez);
+              const int r2 = ex * ex + ey * ey + ez * ez;
+              same |= r2 == 0 ? bit : 0u;
+              sh[0] |= r2 == 3 ? bit : 0u;
+              sh[1] |= NSH > 1 && r2 == 4 ? bit : 0u;
+              sh[2] |= NSH > 2 && r2 == 8 ? bit : 0u;
+              sh[3] |= NSH > 3 && r2 == 11 ? bit : 0u;
+            }
+          };
+          sort_bits(m, ccur, scur, tcur);
+          sort_bits(mb[cur ^ 1], cprev, sprev, tprev);
+          if constexpr (!kSmem) {
+            ccur = scur | tcur[0] | tcur[1] | tcur[2] | tcur[3];
+            cprev = sprev | tprev[0] | tprev[1] | tprev[2] | tprev[3];
+          }
+        }
+        m.head[lane] = make_int4(dq, lu, (int)cprev, (int)ccur);
+        m.place[lane] = make_int4(site, __float_as_int(code.x), __float_as_int(code.y), 0);
+        m.n[lane] = make_float4(nx, ny, nz, __uint_as_float(scur));
+        m.h[lane] = make_float4(hx, hy, hz, __uint_as_float(__brev(sprev)));
+        m.cur[lane] = make_int4((int)tcur[0], (int)tcur[1], (int)tcur[2], (int)tcur[3]);
+        m.prev[lane] = make_int4((int)__brev(tprev[0]), (int)__brev(tprev[1]), (int)__brev(tprev[2]),
+                                 (int)__brev(tprev[3]));
+        const uint32_t touched = __reduce_or_sync(kFullMask, valid ? scur | tcur[0] | tcur[1] | tcur[2] | tcur[3] : 0u);
+        const uint32_t on_site = __reduce_or_sync(kFullMask, valid ? scur : 0u);
+        const int n_long = __popc(__ballot_sync(kFullMask, (unsigned)(dq + (1 << 24)) >= (1u << 25)));
+        if (lane == 0) m.all = make_int4((int)touched, (int)on_site, n_long, 0);
       }
-      r.cprev = b > 0 ? oprev : 0u;
-      r.ccur = ocur & ((1u << lane) - 1u);
-      if constexpr (!kTraj) {
-        const unsigned long long dqu = (unsigned long long)r.dq;
-        pk[cur * 32 + lane] = make_int4((int)(uint32_t)dqu, (int)(uint32_t)(dqu >> 32), (int)r.ccur, r.lu);
-      }
-      r.site = site;
-      r.nx = nx;
-      r.ny = ny;
-      r.nz = nz;
       __syncwarp();
       named_arrive(kBarReady + cur);
       // batch b+1 inserts into the other slot, which still holds batch b-1's bits
@@ -327,39 +372,15 @@ __device__ __forceinline__ void pipe_walk_slot(const WalkerArgs& a, const int sl
   } else if (warp == 0) {
    if constexpr (kTraj) {
     // ------------------------ resolver (trajectory mode) ------------------------
-    double E = 0.0;
-    long long Efx = 0;
-    int bcur;
-    if constexpr (kTraj) {
-      E = a.st.E[slot];
-      bcur = a.st.bin[slot];
-    } else {
-      Efx = a.st.efx[slot];
-      bcur = fx_bin(Efx);
-    }
-    double lnf = 0.0;
-    long long lnf_fx = 0;
-    bool frozen;
-    if constexpr (kTraj) {
-      lnf = a.st.lnf[slot];
-      frozen = !(lnf >= a.lnf_final);
-    } else {
-      lnf_fx = a.st.lnf_fx[slot];
-      frozen = !((double)lnf_fx * kLngUnit >= a.lnf_final);
-    }
+    double E = a.st.E[slot];
+    int bcur = a.st.bin[slot];
+    const double lnf = a.st.lnf[slot];
+    const bool frozen = !(lnf >= a.lnf_final);
     const bool bad = (unsigned)(bcur - wlo) >= (unsigned)W;
     if (bad && lane == 0) atomicExch(a.st.ctrl + 0, kErrOutOfWindow);
-    Lng lng_cur = bad ? Lng(0) : lng_s[bcur - wlo];
+    double lng_cur = bad ? 0.0 : lng_s[bcur - wlo];
     uint32_t h_cur = bad ? 0u : H_s[bcur - wlo];
-    // ln g of the bins next to the current one, kept in registers (production)
-    long long lng_m = 0, lng_p = 0;
-    if constexpr (!kTraj) {
-      if (!bad) {
-        lng_m = bcur - 1 >= wlo ? (long long)lng_s[bcur - 1 - wlo] : 0;
-        lng_p = bcur + 1 < wlo + W ? (long long)lng_s[bcur + 1 - wlo] : 0;
-      }
-    }
-    constexpr int kWords = (int)(sizeof(Rec<kTraj>) / sizeof(int4));
+    constexpr int kWords = (int)(sizeof(TrajRec) / sizeof(int4));
     uint32_t acc_prev = 0;
     long long n_acc = 0, n_rec = 0;
     for (int b = 0; b < nb; ++b) {
@@ -375,7 +396,7 @@ __device__ __forceinline__ void pipe_walk_slot(const WalkerArgs& a, const int sl
         for (int q = 0; q < kWords; ++q) nxt[q] = R4[q];
       }
       for (int k = 0; k < nvalid; ++k) {
-        Rec<kTraj> r;
+        TrajRec r;
         memcpy(&r, nxt, sizeof r);
         if (k + 1 < nvalid) {
 #pragma unroll
@@ -383,79 +404,35 @@ __device__ __forceinline__ void pipe_walk_slot(const WalkerArgs& a, const int sl
         }
         const uint32_t need = (r.cprev & acc_prev) | (r.ccur & acc_cur);
         const int site = r.site;
-        bool acc;
-        if constexpr (kTraj) {
-          double dE = r.dE;
-          if (need) {
-            __syncwarp();
-            int X, Y, Z;
-            bcc_coords(site, L, a.geo.divL, X, Y, Z);
-            double dn = 0.0;
-            if (lane == 0)
-              dn = (double)delta_energy<true>(a, off_s, J_s, lat, site, X, Y, Z, r.nx, r.ny, r.nz, 0, 1, 1u);
-            dE = __shfl_sync(kFullMask, dn, 0);
-            ++n_rec;
-          }
-          const double Ep = __dadd_rn(E, dE);
-          const int bp = bin_fp64(Ep, a.win);
-          const int rel = bp - wlo;
-          acc = false;
-          if ((unsigned)rel < (unsigned)W) {
-            const double lngp = (bp == bcur) ? (double)lng_cur : (double)lng_s[rel];
-            const double d = __dsub_rn((double)lng_cur, lngp);
-            acc = (d >= 0.0) || (r.u < exp_fp64(d, a.ex));
-            if (acc) {
-              if (bp != bcur) {
-                lng_s[bcur - wlo] = lng_cur;
-                H_s[bcur - wlo] = h_cur;
-                lng_cur = (Lng)lngp;
-                h_cur = H_s[rel];
-                bcur = bp;
-              }
-              E = Ep;
+        double dE = r.dE;
+        if (need) {
+          __syncwarp();
+          int X, Y, Z;
+          bcc_coords(site, L, a.geo.divL, X, Y, Z);
+          double dn = 0.0;
+          if (lane == 0)
+            dn = (double)delta_energy<true>(a, off_s, J_s, lat, site, X, Y, Z, r.nx, r.ny, r.nz, 0, 1, 1u);
+          dE = __shfl_sync(kFullMask, dn, 0);
+          ++n_rec;
+        }
+        const double Ep = __dadd_rn(E, dE);
+        const int bp = bin_fp64(Ep, a.win);
+        const int rel = bp - wlo;
+        bool acc = false;
+        if ((unsigned)rel < (unsigned)W) {
+          const double lngp = (bp == bcur) ? lng_cur : lng_s[rel];
+          const double d = __dsub_rn(lng_cur, lngp);
+          acc = (d >= 0.0) || (r.u < exp_fp64(d, a.ex));
+          if (acc) {
+            if (bp != bcur) {
+              lng_s[bcur - wlo] = lng_cur;
+              H_s[bcur - wlo] = h_cur;
+              lng_cur = lngp;
+              h_cur = H_s[rel];
+              bcur = bp;
             }
+            E = Ep;
           }
-        } else {
-          int dq = r.dq;
-          if (need) {
-            __syncwarp();
-            int X, Y, Z;
-            bcc_coords(site, L, a.geo.divL, X, Y, Z);
-            const float dEn = (float)delta_energy<false>(a, off_s, J_s, lat, site, X, Y, Z, r.nx, r.ny, r.nz,
-                                                         lane, 32, kFullMask);
-            dq = dq24_of(dEn, a.win);
-            ++n_rec;
-          }
-          const long long Ep = Efx + ((long long)dq << 8);
-          const int bp = fx_bin(Ep);
-          const int db = bp - bcur;
-          if (db == 0) {
-            acc = true;                      // same bin: ln g ratio 1
-          } else {
-            const int rel = bp - wlo;
-            acc = false;
-            if ((unsigned)rel < (unsigned)W) {
-              const long long lngp = db == 1 ? lng_p : (db == -1 ? lng_m : (long long)lng_s[rel]);
-              const long long d = (long long)lng_cur - lngp;
-              const int d20 = d < -(1LL << 51) ? (int)0x80000000 : (int)(d >> 20);
-              acc = d >= 0 || r.lu < d20;
-              if (acc) {
-                lng_s[bcur - wlo] = lng_cur;
-                H_s[bcur - wlo] = h_cur;
-                if (db == 1) {
-                  lng_m = (long long)lng_cur;
-                } else if (db == -1) {
-                  lng_p = (long long)lng_cur;
-                }
-                lng_cur = (Lng)lngp;
-                h_cur = H_s[rel];
-                bcur = bp;
-                if (db != -1) lng_p = bcur + 1 < wlo + W ? (long long)lng_s[bcur + 1 - wlo] : 0;
-                if (db != 1) lng_m = bcur - 1 >= wlo ? (long long)lng_s[bcur - 1 - wlo] : 0;
-              }
-            }
-          }
-          if (acc) Efx = Ep;
         }
         if (acc) {
           acc_cur |= 1u << k;
@@ -463,10 +440,7 @@ __device__ __forceinline__ void pipe_walk_slot(const WalkerArgs& a, const int sl
           if (lane == 0) lat.set(site, r.nx, r.ny, r.nz);
         }
         if (!frozen) {
-          if constexpr (kTraj)
-            lng_cur = (Lng)__dadd_rn((double)lng_cur, lnf);
-          else
-            lng_cur = (Lng)((long long)lng_cur + lnf_fx);
+          lng_cur = __dadd_rn(lng_cur, lnf);
           ++h_cur;
         }
       }
@@ -475,12 +449,8 @@ __device__ __forceinline__ void pipe_walk_slot(const WalkerArgs& a, const int sl
       named_arrive(kBarDone + cur);
     }
     if (lane == 0 && !bad) {
-      if constexpr (kTraj) {
-        a.st.E[slot] = E;
-        a.st.bin[slot] = bcur;
-      } else {
-        a.st.efx[slot] = Efx;
-      }
+      a.st.E[slot] = E;
+      a.st.bin[slot] = bcur;
       lng_s[bcur - wlo] = lng_cur;
       H_s[bcur - wlo] = h_cur;
       a.st.steps[slot] = t0 + moves;
@@ -492,14 +462,19 @@ __device__ __forceinline__ void pipe_walk_slot(const WalkerArgs& a, const int sl
     // The lattice holds every batch up to b-2 while batch b is resolved: batch b-1's accepted spins
     // are written at the start of batch b, after the producer has read the lattice for batch b.  A
     // move's energy change then follows exactly from the producer's snapshot (field h, old spin o)
-    // and the accepted moves of batch b-1 and of batch b before it that touch its neighbourhood:
-    // each adds J (S' - S) to h, or replaces o when it sits on the move's own site.  Corrections
-    // from batch b-1 are applied by every lane at the start of the batch; those from batch b are
-    // out-of-line events of the sequential part.
-    // Current bin: its ln g and H stay in registers and are written back only when the walker
-    // leaves the bin; ln g of the two neighbouring bins is cached (lng_m, lng_p).
-    long long Efx = a.st.efx[slot];
-    int bcur = fx_bin(Efx);
+    // and the accepted moves of batch b-1 and of batch b before it that touch it: each adds
+    // J (S' - S) to h, or replaces o when it sits on the move's own site, in the order of the moves.
+    // Lane k holds move k throughout: it pulls the corrections from batch b-1 at the start, and when a
+    // move of this batch is accepted, every later lane that it touches takes its correction at once
+    // (push), all lanes together.
+    // The walker's state is its bin r of the window and the fraction of the bin below its energy, in
+    // 2^-24 bins (the eight lowest bits of the fixed-point energy never change during a walk: increments
+    // are whole 2^-24 bins).  ln g of the current bin at move k is A + k ln f; it goes back to the table
+    // only when the walker leaves the bin.
+    const long long efx0 = a.st.efx[slot];
+    int r = fx_bin(efx0) - wlo;
+    int frac = (int)((uint32_t)efx0 >> 8);
+    const uint32_t frac_low = (uint32_t)efx0 & 0xffu;
     // shell couplings as four scalars: an indexed read of the parameter array would be a
     // constant-memory load whose lanes take different indexes, serialised lane by lane
     const float J0 = a.geo.Jsh_f[0], J1 = NSH > 1 ? a.geo.Jsh_f[1] : 0.0f, J2 = NSH > 2 ? a.geo.Jsh_f[2] : 0.0f,
@@ -507,392 +482,426 @@ __device__ __forceinline__ void pipe_walk_slot(const WalkerArgs& a, const int sl
     const long long lnf_fx = a.st.lnf_fx[slot];
     const bool frozen = !((double)lnf_fx * kLngUnit >= a.lnf_final);
     const long long lnf_eff = frozen ? 0 : lnf_fx;
-    const uint32_t hinc = frozen ? 0u : 1u;
-    const bool bad = (unsigned)(bcur - wlo) >= (unsigned)W;
-    if (bad && lane == 0) atomicExch(a.st.ctrl + 0, kErrOutOfWindow);
-    long long lng_in = bad ? 0 : (long long)lng_s[bcur - wlo];
-    uint32_t h_in = bad ? 0u : H_s[bcur - wlo];
-    long long lng_m = 0, lng_p = 0;
-    if (!bad) {
-      lng_m = bcur - 1 >= wlo ? (long long)lng_s[bcur - 1 - wlo] : 0;
-      lng_p = bcur + 1 < wlo + W ? (long long)lng_s[bcur + 1 - wlo] : 0;
+    const bool bad = (unsigned)r >= (unsigned)W;
+    if (bad) {
+      if (lane == 0) atomicExch(a.st.ctrl + 0, kErrOutOfWindow);
+      r = 0;                                // no move is made
     }
-    // coupling between sites p and q: J of q's shell around p, 0 if q is not a neighbour (every
-    // offset component is below L half-units, so the wrapped displacement is the offset itself)
-    auto coupling = [&](int p, int q) -> float {
-      int Xp, Yp, Zp, Xq, Yq, Zq;
-      bcc_coords(p, L, a.geo.divL, Xp, Yp, Zp);
-      bcc_coords(q, L, a.geo.divL, Xq, Yq, Zq);
-      int dx = Xq - Xp, dy = Yq - Yp, dz = Zq - Zp;
-      dx += dx < -L ? 2 * L : 0;
-      dx -= dx >= L ? 2 * L : 0;
-      dy += dy < -L ? 2 * L : 0;
-      dy -= dy >= L ? 2 * L : 0;
-      dz += dz < -L ? 2 * L : 0;
-      dz -= dz >= L ? 2 * L : 0;
-      // squared half-unit distances 3, 4, 8, 11 are the shells 1..4
-      const int r2 = dx * dx + dy * dy + dz * dz;
-      return r2 == 3 ? J0 : (r2 == 4 ? J1 : (r2 == 8 ? J2 : (r2 == 11 ? J3 : 0.0f)));
-    };
-    // field and old spin of a move at site p after the accepted moves m of record block R, in order;
-    // returns the moves among m that sit on site p (a later accepted move supersedes them)
-    auto correct = [&](const Rec<false>* R, uint32_t m, int p, float& hx, float& hy, float& hz, float& ox, float& oy,
-                       float& oz) -> uint32_t {
-      uint32_t same = 0u;
-      while (m) {
-        const int j = __ffs(m) - 1;
-        m &= m - 1u;
-        const Rec<false>& rj = R[j];
-        const int q = rj.site;
-        if (q == p) {
-          ox = rj.nx;
-          oy = rj.ny;
-          oz = rj.nz;
-          same |= 1u << j;
-        } else {
-          const float J = coupling(p, q);
-          hx = fmaf(J, rj.dsx, hx);
-          hy = fmaf(J, rj.dsy, hy);
-          hz = fmaf(J, rj.dsz, hz);
-        }
-      }
-      return same;
-    };
-    // write the accepted spins of record block R: acc minus the moves superseded on their site
-    auto publish = [&](const Rec<false>* R, uint32_t acc) {
-      if ((acc >> lane) & 1u) {
-        const Rec<false>& rp = R[lane];
-        lat.set_code(rp.site, make_float2(rp.cu, rp.cv));
-      }
-      __syncwarp();
-    };
-    // segment state: the walker entered bcur (or the batch began) at move k_seg with ln g = lng_seg
-    // and histogram h_seg; after j more moves there, ln g = lng_seg + j ln f
-    long long lng_seg = lng_in;
-    uint32_t h_seg = h_in;
-    uint32_t acc_prev = 0, pub_prev = 0;
-    int n_rec = 0;
-    long long n_acc = 0;
-    // Three ways through a batch, all with the same decisions; each batch takes the cheapest for
-    // the counts of the batch before it: n_rej moves that left the bin to a neighbour and were
-    // rejected, n_ev moves resolved out of line (accepted bin changes, jumps of two or more bins,
-    // corrections).
-    //   scan       -- one warp scan, one ballot round per event: few events (high-energy windows);
-    //   blocks     -- branch-free blocks of 8 moves absorb rejected exits: many of those, few others
-    //                 (low-energy windows);
-    //   sequential -- one move at a time: many full resolutions (bins as narrow as the temperature).
+    long long A = (long long)lng_s[r];
+    const long long lane_lnf = (long long)lane * lnf_eff;
+    constexpr int kBin = 1 << 24;
+    constexpr uint32_t kNoKey = 0xffffffffu;
+    constexpr int kDense = 14;
+    const uint32_t lane_key = (uint32_t)lane << 27;
+    // Three ways through a batch, all with the same decisions; each batch takes the cheapest for the
+    // counts of the batch before it:
+    //   scan       -- a run of moves that stay in the bin is accepted together; one round per move that
+    //                 leaves it: few exits (high-energy windows);
+    //   blocks     -- one round per accepted move, steps to a neighbouring bin decided by two pass bits
+    //                 per move: few accepted moves, few bin changes (low-energy windows, where most
+    //                 proposals are rejected exits);
+    //   sequential -- one round per accepted move, every lane looking up ln g at its own target bin: any
+    //                 accepted move may change bin (bins as narrow as the temperature).
+    // What bounds it: the chain from one accepted move to the next, latency alone (one warp, every
+    // instruction waits for the one before).  So a round costs as few dependent steps as possible, and
+    // rejected moves cost nothing.  Resolving one move after the other, or blocks of 8 with a restart at
+    // every event, took 90-350 cycles per move; now (ms per 10^4 moves, GB300) bcc L = 16, 2 shells,
+    // [E_gs, 0], 64 walkers: 0.69 -> 0.47; bcc L = 8, 3 shells, converging (4000 moves): 1.03 -> 0.49;
+    // 576 walkers of bcc L = 4, 5, 6, converging (4000 moves): 3.1 -> 0.66.
+    // A round finds the first move that counts, and what it does, with one warp minimum (24 cycles; a
+    // vote, a find-first-set and a shuffle take 100): key = lane << 27 | payload, all ones for lanes
+    // with nothing to say and for decided moves.  One branch per round tells the rare payloads apart.
     enum { kScan = 0, kBlocks = 1, kSequential = 2 };
-    // several sites share an owner entry (lattices in global memory; a shared-memory lattice keeps
-    // its walker's code as it is, which measured faster at bcc L = 16 where its table has an entry
-    // per site)
-    const bool aliased = !kSmem && (long long)omask + 1 < (long long)N;
     const int forced = a.resolver - 1;      // -1: per-batch choice
-    int path = forced >= 0 ? forced : kBlocks;
+    int path = kBlocks, n_in = 0, n_exit = 32, n_chg = 0;
     int n_scan = 0, n_blocks = 0, n_seq = 0;   // batches per path
+    uint32_t acc_prev = 0, acc_prev_rev = 0, pub_prev = 0;
+    int4 place_prev = make_int4(0, 0, 0, 0);
+    long long n_acc = 0;
+    unsigned n_rec = 0;                        // this lane's corrected moves
     for (int b = 0; b < nb; ++b) {
       const int cur = b & 1;
       named_sync(kBarReady + cur);
       const int nvalid = bad ? 0 : (int)(moves - (long long)b * 32 < 32 ? moves - (long long)b * 32 : 32);
-      int k_seg = 0;
-      uint32_t acc_cur = 0, sup = 0;
-      int n_rej = 0, n_ev = 0;
-      Rec<false>* Rc = rec + cur * 32;
-      const Rec<false>* Rp = rec + (cur ^ 1) * 32;
-      // ---- parallel part: lane = move index ----
-      Rec<false>& mine = Rc[lane];
+      const bool valid = lane < nvalid;
+      MoveBatch& C = mb[cur];
+      const MoveBatch& P = mb[cur ^ 1];
+      const int4 all = C.all;
+      const int4 hd = C.head[lane];
+      const float4 n4 = C.n[lane];
+      float4 h4 = C.h[lane], d4 = C.ds[lane];
+      const int4 tc = C.cur[lane], tp = C.prev[lane];
+      const uint32_t touched = (uint32_t)all.x;     // moves that touch a later one
+      const uint32_t sc = __float_as_uint(n4.w);
+      const int4 place = C.place[lane];
+      int dq = hd.x;
+      auto increment = [&]() { dq = dq24_of(-fmaf(d4.z, h4.z, fmaf(d4.y, h4.y, d4.x * h4.x)), a.win); };
+      // coupling of the shell whose mask has this bit
+      auto coupling = [&](const int4& t, uint32_t bit) -> float {
+        float J = (uint32_t)t.x & bit ? J0 : 0.0f;
+        if constexpr (NSH > 1) J = (uint32_t)t.y & bit ? J1 : J;
+        if constexpr (NSH > 2) J = (uint32_t)t.z & bit ? J2 : J;
+        if constexpr (NSH > 3) J = (uint32_t)t.w & bit ? J3 : J;
+        return J;
+      };
+      // an accepted move with proposed spin v sits on this lane's site
+      auto replace = [&](const float4 v) {
+        d4.x = n4.x - v.x;
+        d4.y = n4.y - v.y;
+        d4.z = n4.z - v.z;
+        C.ds[lane] = d4;
+      };
+      // ---- corrections from batch b-1 ----
       {
-        // An owner table smaller than the lattice is hashed, so a conflict bit may name a move whose
-        // site is neither this move's site nor one of its neighbours: such a move cannot change this
-        // move's field or old spin.  Drop those bits once here -- from batch b-1 (accepted moves)
-        // and from this batch (before any is resolved) -- so that only real conflicts become events
-        // below.  (At bcc L = 32 with 2048 entries, 92 % of the flagged moves were such aliases.)
-        uint32_t m = lane < nvalid ? (mine.cprev & acc_prev) : 0u;
-        const uint32_t cc = (lane < nvalid && aliased) ? mine.ccur : 0u;
-        if (aliased && (m | cc)) {
-          const int p0 = mine.site;
-          uint32_t real_prev = 0u, real_cur = 0u;
-          for (uint32_t t = m; t; t &= t - 1u) {
-            const int j = __ffs(t) - 1;
-            const int q = Rp[j].site;
-            if (q == p0 || coupling(p0, q) != 0.0f) real_prev |= 1u << j;
-          }
-          for (uint32_t t = cc; t; t &= t - 1u) {
-            const int j = __ffs(t) - 1;
-            const int q = Rc[j].site;
-            if (q == p0 || coupling(p0, q) != 0.0f) real_cur |= 1u << j;
-          }
-          m = real_prev;
-          if (real_cur != cc) pk[cur * 32 + lane].z = (int)real_cur;
+        const uint32_t sp = __float_as_uint(h4.w);
+        uint32_t t = valid ? (sp | (uint32_t)tp.x | (uint32_t)tp.y | (uint32_t)tp.z | (uint32_t)tp.w) & acc_prev_rev : 0u;
+        n_rec += valid && ((uint32_t)hd.z & acc_prev) != 0u ? 1u : 0u;
+        if (t) {
+          do {
+            const int j = __clz((int)t);
+            const uint32_t bit = 0x80000000u >> j;
+            t ^= bit;
+            const float4 dj = P.ds[j];
+            if (sp & bit) {
+              replace(P.n[j]);
+            } else {
+              const float J = coupling(tp, bit);
+              h4.x = fmaf(J, dj.x, h4.x);
+              h4.y = fmaf(J, dj.y, h4.y);
+              h4.z = fmaf(J, dj.z, h4.z);
+            }
+          } while (t);
+          increment();
         }
-        // accepted moves of batch b-1 around this move: correct h and o, then dE
-        if (m) {
-          float hx = mine.hx, hy = mine.hy, hz = mine.hz, ox = mine.ox, oy = mine.oy, oz = mine.oz;
-          correct(Rp, m, mine.site, hx, hy, hz, ox, oy, oz);
-          const float dx = mine.nx - ox, dy = mine.ny - oy, dz = mine.nz - oz;
-          const float dE = -fmaf(dz, hz, fmaf(dy, hy, dx * hx));
-          const long long dq = (long long)dq24_of(dE, a.win) << 8;
-          mine.dq = dq;
-          mine.hx = hx;
-          mine.hy = hy;
-          mine.hz = hz;
-          mine.ox = ox;
-          mine.oy = oy;
-          mine.oz = oz;
-          mine.dsx = dx;
-          mine.dsy = dy;
-          mine.dsz = dz;
-          const unsigned long long dqu = (unsigned long long)dq;
-          pk[cur * 32 + lane].x = (int)(uint32_t)dqu;
-          pk[cur * 32 + lane].y = (int)(uint32_t)(dqu >> 32);
-        }
-        n_rec += __popc(__ballot_sync(kFullMask, m != 0u));
       }
-      // batch b-1's spins go to the lattice now that the producer has read it for batch b
+      // batch b-1's spins go to the lattice now that the producer has read it for batch b: accepted
+      // moves, minus those superseded on their site
       if (b > 0) {
-        publish(Rp, pub_prev);
-        named_arrive(kBarDone + (cur ^ 1));
-      } else {
+        if ((pub_prev >> lane) & 1u)
+          lat.set_code(place_prev.x, make_float2(__int_as_float(place_prev.y), __int_as_float(place_prev.z)));
         __syncwarp();
+        named_arrive(kBarDone + (cur ^ 1));
       }
-      const int my_lu = mine.lu;
-      // would a step to bcur + 1 / bcur - 1 be accepted at this move, given no change of bin since
-      // k_seg (lane = move; ln g at move k is lng_seg + (k - k_seg) ln f)
-      auto pass_masks = [&](uint32_t& up, uint32_t& down) {
-        const long long ln = lng_seg + (long long)(lane - k_seg) * lnf_eff;
-        const long long du = ln - lng_p, dd = ln - lng_m;
-        const int u20 = du < -(1LL << 51) ? (int)0x80000000 : (int)(du >> 20);
-        const int l20 = dd < -(1LL << 51) ? (int)0x80000000 : (int)(dd >> 20);
-        const bool pu = bcur + 1 < wlo + W && (du >= 0 || my_lu < u20);
-        const bool pd = bcur - 1 >= wlo && (dd >= 0 || my_lu < l20);
-        up = __ballot_sync(kFullMask, pu);
-        down = __ballot_sync(kFullMask, pd);
+      place_prev = place;
+      // ---- the batch in order ----
+      // Measured (cycles per batch): blocks 350 + 95 per accepted move + 350 per bin change (and per move
+      // of a bin or more, if undecided by the pass bits), scan 450 + 100 per rejected exit + 300 per other
+      // event, sequential 300 + 160 per accepted move (250 where every accepted move is pushed).  So two
+      // bin changes, or two moves that may reach beyond the next bin, make the sequential path the
+      // cheaper one; between the other two the counts of exits and of accepted moves decide.
+      path = forced >= 0 ? forced
+                         : (n_chg >= 2 || all.z >= 2 ? kSequential : (n_exit + 2 < n_in ? kScan : kBlocks));
+      uint32_t same = 0u;                  // accepted moves of this batch on this lane's site
+      uint32_t acc_cur = 0u;
+      int rb = r;                          // bin before this lane's move
+      n_chg = 0;                           // bin changes
+      // A move is accepted iff ln g(now) - ln g(target) >= T, T = min(0, (ln u + 1) 2^20): with
+      // d = ln g(now) - ln g(target) in 2^-40 units this is d >= 0 or ln u < floor(d / 2^20).  With
+      // ln g(now) = A + lane ln f: ln g(target) <= A + Q.
+      const long long Q = lane_lnf - (hd.y < 0 ? (long long)(hd.y + 1) * 1048576LL : 0LL);
+      auto push = [&](const int e) {
+        const uint32_t bit = 1u << e;
+        const float4 de = C.ds[e];
+        const float J = coupling(tc, bit);
+        h4.x = fmaf(J, de.x, h4.x);        // J = 0: unchanged
+        h4.y = fmaf(J, de.y, h4.y);
+        h4.z = fmaf(J, de.z, h4.z);
+        const float4 v = C.n[e];
+        const bool own = (sc & bit) != 0u;   // it sits on this lane's site
+        d4.x = own ? n4.x - v.x : d4.x;
+        d4.y = own ? n4.y - v.y : d4.y;
+        d4.z = own ? n4.z - v.z : d4.z;
+        if (own) C.ds[lane] = d4;
+        same |= sc & bit;
+        increment();
       };
-      // One move kk with increment dq (corrected first if it meets an accepted move of this batch):
-      // Metropolis step on ln g, bin bookkeeping; every lane computes the same values.  Returns
-      // whether the walker changed bin.
-      auto resolve = [&](const int kk, long long dq, const uint32_t ccur_w, const int lu) -> bool {
-        const uint32_t m = ccur_w & acc_cur;
-        uint32_t same = 0u;
-        if (m) {
-          Rec<false>& rk = Rc[kk];
-          float hx = rk.hx, hy = rk.hy, hz = rk.hz, ox = rk.ox, oy = rk.oy, oz = rk.oz;
-          same = correct(Rc, m, rk.site, hx, hy, hz, ox, oy, oz);
-          const float dx = rk.nx - ox, dy = rk.ny - oy, dz = rk.nz - oz;
-          const float dEn = -fmaf(dz, hz, fmaf(dy, hy, dx * hx));
-          dq = (long long)dq24_of(dEn, a.win) << 8;
-          __syncwarp();
-          if (lane == 0) {
-            rk.dsx = dx;
-            rk.dsy = dy;
-            rk.dsz = dz;
-          }
-          __syncwarp();
-          ++n_rec;
-        }
-        const long long Ep = Efx + dq;
-        const int db = fx_bin(Ep) - bcur;
-        bool acc = true, moved = false;
-        if (db != 0) {
-          const int bp = bcur + db;
-          const int rel = bp - wlo;
-          acc = false;
-          if ((unsigned)rel < (unsigned)W) {
-            const long long lng_now = lng_seg + (long long)(kk - k_seg) * lnf_eff;
-            const long long lngp = db == 1 ? lng_p : (db == -1 ? lng_m : (long long)lng_s[rel]);
-            const long long d = lng_now - lngp;
-            const int e20 = d < -(1LL << 51) ? (int)0x80000000 : (int)(d >> 20);
-            acc = d >= 0 || lu < e20;
-            moved = acc;
-            if (acc) {
-              // leave bcur: write it back, shift the neighbour cache, start a new segment
-              lng_s[bcur - wlo] = (Lng)lng_now;
-              H_s[bcur - wlo] = h_seg + hinc * (uint32_t)(kk - k_seg);
-              if (db == 1) lng_m = lng_now;
-              if (db == -1) lng_p = lng_now;
-              lng_seg = lngp;
-              h_seg = H_s[rel];
-              k_seg = kk;
-              bcur = bp;
-              if (db != -1) lng_p = bcur + 1 < wlo + W ? (long long)lng_s[bcur + 1 - wlo] : 0;
-              if (db != 1) lng_m = bcur - 1 >= wlo ? (long long)lng_s[bcur - 1 - wlo] : 0;
-            }
-          }
-        }
-        if (acc) {
-          Efx = Ep;
-          acc_cur |= 1u << kk;
-          sup |= same;   // earlier accepted moves on this site are no longer the site's spin
-        }
-        const bool neighbour_reject = !acc && (db == 1 || db == -1) && !m;
-        n_rej += neighbour_reject ? 1 : 0;
-        n_ev += (db != 0 && !neighbour_reject) || m ? 1 : 0;
-        return moved;
+      // the accepted move e leaves the bin for bin r + db
+      auto change_bin = [&](const int e, const int db) {
+        const long long el = (long long)e * lnf_eff;
+        lng_s[r] = (Lng)(A + el);
+        r += db;
+        A = (long long)lng_s[r] - el;
+        rb = lane > e ? r : rb;
+        ++n_chg;
       };
-      // ---- sequential part as a scan ----
-      // A move that stays in the current bin is accepted (ln g ratio 1), so between events the
-      // energy is a running sum: with P_k the inclusive prefix sum of the batch's increments and
-      // segment base B (fraction before move s minus the prefix before s), move k >= s lands at
-      // fraction B + P_k.  The first move that leaves [0, 2^32) -- or meets an accepted move of this
-      // batch -- ends the segment: the moves before it stand.  A step to a neighbouring bin whose
-      // pass bit is clear is rejected on the spot (the base drops its increment); anything else is
-      // resolved on its own.  One scan per batch, one round of ballots per such move.
-      const int4* P4 = pk + cur * 32;
-      uint32_t up_mask = 0, down_mask = 0;
-      if (path == kScan && nvalid > 0) {
-        const int4 wk = P4[lane];
-        const long long dqk = lane < nvalid ? (long long)(((unsigned long long)(uint32_t)wk.y << 32) | (uint32_t)wk.x)
-                                            : 0LL;
-        long long P = dqk;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          const long long t = __shfl_up_sync(kFullMask, P, o);
-          if (lane >= o) P += t;
-        }
-        const uint32_t cck = (uint32_t)wk.z;
-        const uint32_t below = (1u << lane) - 1u;          // moves before this one
-        const uint32_t upto = nvalid >= 32 ? 0xffffffffu : ((1u << nvalid) - 1u);
-        pass_masks(up_mask, down_mask);
-        long long B = (long long)(uint32_t)Efx;
-        int s0 = 0;
+      // Would a step to bin r + 1 / r - 1 be accepted at this lane's move: positions [lo, lo + span)
+      // (2^-24 bins from the bottom of bin r) are accepted, those inside the bin among them.
+      int lo = 0;
+      uint32_t span = 0;
+      auto pass = [&]() {
+        const bool up = r + 1 < W && (long long)lng_s[min(r + 1, W - 1)] <= A + Q;
+        const bool down = r > 0 && (long long)lng_s[max(r - 1, 0)] <= A + Q;
+        lo = down ? -kBin : 0;
+        span = (uint32_t)(kBin + (up ? kBin : 0) - lo);
+      };
+      // the target bin r + db of move e, looked up
+      auto admits = [&](const int e, const int db) -> bool {
+        return (unsigned)(r + db) < (unsigned)W && (long long)lng_s[r + db] <= A + shfl_ll(Q, e);
+      };
+      if (path == kSequential && __popc(touched) >= kDense) {
+        // Many moves touch a later one (small lattices): every round pushes, without asking.  Measured,
+        // ms per 10^4 moves with and without this form: 1.03 and 1.36 at bcc L = 4 (about 27 of 32 moves
+        // touch a later one), 1.26 and 1.21 at L = 8 (11 of 32).
+        // payload: the increment, -4..4 bins; kRare (-4 bins) stands for a longer one, and for -1 (whose
+        // key would be kNoKey in lane 31).
+        constexpr uint32_t kRare = 0x04000000u, kPayload = 0x07ffffffu;
+        bool live = valid;
         while (true) {
-          const uint32_t from_s = ~((1u << s0) - 1u);      // moves s0 .. 31
-          const long long pos = B + P;
-          const bool live = lane >= s0 && lane < nvalid;
-          const uint32_t outs = __ballot_sync(kFullMask, live && (unsigned long long)pos >= (1ull << 32));
-          const uint32_t needs = __ballot_sync(kFullMask, live && (cck & (acc_cur | (below & from_s))) != 0u);
-          const uint32_t ev = outs | needs;
-          if (ev == 0u) {
-            // the rest of the batch stays in the bin
-            acc_cur |= upto & from_s;
-            const long long Pl = __shfl_sync(kFullMask, P, nvalid - 1);
-            Efx = ((long long)bcur << 32) | (long long)(uint32_t)(B + Pl);
-            break;
+          const int pos = frac + dq, rel = r + (pos >> 24);
+          const long long lt = (long long)lng_s[min((unsigned)rel, (unsigned)W - 1u)];
+          const bool plain = (unsigned)(dq + 4 * kBin - 1) < 8u * kBin - 1u && dq != -1;
+          const uint32_t key = lane_key | (plain ? (uint32_t)dq & kPayload : kRare);
+          // ln g of the walker's own bin in the table is at most its present value, so a move that
+          // stays passes the test too
+          const bool ok = live && (unsigned)rel < (unsigned)W && lt <= A + Q;
+          const uint32_t m = __reduce_min_sync(kFullMask, ok ? key : kNoKey);
+          const int e = (int)(m >> 27);
+          const long long A2 = shfl_ll(rel == r ? A : lt - lane_lnf, e);   // ln g after the move, less e ln f
+          int pe = frac + ((int)(m << 5) >> 5);
+          if ((m & kPayload) == kRare || m == kNoKey) {
+            if (m == kNoKey) break;        // every move left is rejected
+            pe = __shfl_sync(kFullMask, pos, e);
           }
-          const int e = __ffs(ev) - 1;
-          const uint32_t bit = 1u << e;
-          acc_cur |= (bit - 1u) & from_s;
-          const long long pe = __shfl_sync(kFullMask, pos, e);
-          const long long de = __shfl_sync(kFullMask, dqk, e);
-          if (!(needs & bit)) {
-            // leaves the bin: one bin up or down with the pass bit clear is rejected here
-            const bool one_up = pe >= (1LL << 32) && pe < (2LL << 32);
-            const bool one_down = pe < 0 && pe >= -(1LL << 32);
-            if ((one_up && !(up_mask & bit)) || (one_down && !(down_mask & bit))) {
-              ++n_rej;
-              B -= de;
-              s0 = e + 1;
-              if (s0 >= nvalid) {
-                Efx = ((long long)bcur << 32) | (long long)(uint32_t)(pe - de);
-                break;
-              }
-              continue;
-            }
-          }
-          Efx = ((long long)bcur << 32) | (long long)(uint32_t)(pe - de);
-          const int4 we = P4[e];
-          const long long dq = (long long)(((unsigned long long)(uint32_t)we.y << 32) | (uint32_t)we.x);
-          if (resolve(e, dq, (uint32_t)we.z, we.w)) pass_masks(up_mask, down_mask);
-          s0 = e + 1;
-          if (s0 >= nvalid) break;
-          B = (long long)(uint32_t)Efx - (pe - B);
+          lng_s[r] = (Lng)(A + (long long)e * lnf_eff);
+          n_chg += (pe >> 24) != 0 ? 1 : 0;
+          r += pe >> 24;
+          frac = pe & (kBin - 1);
+          A = A2;
+          acc_cur |= 1u << e;
+          live = live && lane > e;
+          rb = lane > e ? r : rb;
+          push(e);
         }
       } else if (path == kSequential) {
-        // ---- sequential part, one move at a time ----
-        int4 w = P4[0];
-        for (int kk = 0; kk < nvalid; ++kk) {
-          const int4 wn = P4[(kk + 1) & 31];
-          const long long dq = (long long)(((unsigned long long)(uint32_t)w.y << 32) | (uint32_t)w.x);
-          resolve(kk, dq, (uint32_t)w.z, w.w);
-          w = wn;
-        }
-      } else {
-        // ---- sequential part, in branch-free blocks of 8 moves ----
-        // Within a bin the state is frac = Efx - (bcur << 32) in [0, 2^32).  A move in the same bin
-        // is accepted (frac += dq); a step to a neighbouring bin is accepted iff its pass bit is
-        // set, an event handled out of line, like moves that meet an accepted move of this batch
-        // and jumps of two or more bins.  The common path uses no compare-and-select: masks come
-        // from sign bits.
-        pass_masks(up_mask, down_mask);
-        uint32_t frac = (uint32_t)Efx;
-        int k = 0;
-        while (k < nvalid) {
-          const uint32_t acc0 = acc_cur;
-          uint32_t exc = 0, outb = 0;
-          uint32_t fh[8];   // fraction before each move of the block, for the restart
-          int4 q[8];
-#pragma unroll
-          for (int u = 0; u < 8; ++u) q[u] = P4[(k + u) & 31];
-#pragma unroll
-          for (int u = 0; u < 8; ++u) {
-            const int kk = k + u;
-            fh[u] = frac;
-            const uint32_t lo = (uint32_t)q[u].x;
-            const int hi = q[u].y;
-            const uint32_t cc = (uint32_t)q[u].z;
-            const uint32_t vmask = (uint32_t)((kk - nvalid) >> 31);          // all ones while kk < nvalid
-            const uint32_t bit = (1u << (kk & 31)) & vmask;
-            const uint32_t t_lo = frac + lo;
-            const uint32_t carry = ((frac & lo) | ((frac | lo) & ~t_lo)) >> 31;
-            const int th = hi + (int)carry;                                     // high word of frac + dq: bins moved
-            const uint32_t nz = (uint32_t)((th | -th) >> 31);                   // all ones iff th != 0
-            const uint32_t stay = ~nz & vmask;
-            frac = (t_lo & stay) | (frac & ~stay);
-            acc_cur |= bit & stay;
-            outb |= bit & nz;
-            const uint32_t up = (uint32_t)(((th - 1) | (1 - th)) >> 31);       // all ones iff th != 1
-            const uint32_t dn = (uint32_t)(((th + 1) | (-1 - th)) >> 31);      // all ones iff th != -1
-            const uint32_t far = nz & up & dn;                                  // |th| >= 2
-            const uint32_t need = cc & acc_cur & ~bit;
-            exc |= bit & (((~up) & up_mask) | ((~dn) & down_mask) | far | (need ? 0xffffffffu : 0u));
+        // payload: the increment, -4..4 bins; kRare (-4 bins) stands for a longer one, for -1 (whose key
+        // would be kNoKey in lane 31) and for a move that touches a later one.
+        // pos, at: positions relative to bin r0, which follows the walker when it is 16 bins away (sums
+        // stay below 128 bins).
+        constexpr uint32_t kRare = 0x04000000u, kPayload = 0x07ffffffu;
+        int r0 = r, at = frac;
+        auto make_key = [&]() -> uint32_t {
+          const bool plain = (unsigned)(dq + 4 * kBin - 1) < 8u * kBin - 1u && dq != -1 && !((touched >> lane) & 1u);
+          return lane_key | (plain ? (uint32_t)dq & kPayload : kRare);
+        };
+        uint32_t key = valid ? make_key() : kNoKey;
+        int pos, rel;
+        long long lt;
+        auto look = [&]() {
+          pos = at + dq;
+          rel = r0 + (pos >> 24);
+          lt = (long long)lng_s[min((unsigned)rel, (unsigned)W - 1u)];
+        };
+        look();
+        bool away = false;
+        while (true) {
+          // ln g of the walker's own bin in the table is at most its present value, so a move that
+          // stays passes the test too
+          const bool ok = (unsigned)rel < (unsigned)W && lt <= A + Q;
+          const uint32_t m = __reduce_min_sync(kFullMask, ok ? key : kNoKey);
+          const int e = (int)(m >> 27);
+          const long long A2 = shfl_ll(rel == r ? A : lt - lane_lnf, e);   // ln g after the move, less e ln f
+          const bool rare = (m & kPayload) == kRare || m == kNoKey || away;
+          const int at2 = at + ((int)(m << 5) >> 5);
+          if (!rare) lng_s[r] = (Lng)(A + (long long)e * lnf_eff);
+          const int pos2 = at2 + dq, rel2 = r0 + (pos2 >> 24);
+          const long long lt2 = (long long)lng_s[min((unsigned)rel2, (unsigned)W - 1u)];
+          int rn;
+          if (rare) {
+            if (m == kNoKey) break;        // every move left is rejected
+            const int pe = __shfl_sync(kFullMask, pos, e);
+            lng_s[r] = (Lng)(A + (long long)e * lnf_eff);
+            r0 += pe >> 24;
+            at = pe & (kBin - 1);
+            rn = r0;
+            key = lane > e ? key : kNoKey;
+            if ((touched >> e) & 1u) {
+              push(e);
+              key = key == kNoKey ? kNoKey : make_key();
+            }
+            look();
+          } else {
+            at = at2;
+            pos = pos2;
+            rel = rel2;
+            lt = lt2;
+            rn = r0 + (at >> 24);
+            key = lane > e ? key : kNoKey;
           }
-          if (exc == 0u) {
-            n_rej += __popc(outb);
-            k += 8;
-            continue;
-          }
-          n_rej += __popc(outb & ((exc & (0u - exc)) - 1u));
-          // first exceptional move: the block's moves before it stand; restore the state there
-          const int kx = __ffs(exc) - 1;
-#pragma unroll
-          for (int u = 0; u < 8; ++u)
-            if (k + u == kx) frac = fh[u];
-          acc_cur = acc0 | (acc_cur & ((1u << kx) - 1u));
-          Efx = ((long long)bcur << 32) | frac;
-          const int4 wx = P4[kx];
-          const long long dq = (long long)(((unsigned long long)(uint32_t)wx.y << 32) | (uint32_t)wx.x);
-          if (resolve(kx, dq, (uint32_t)wx.z, wx.w)) pass_masks(up_mask, down_mask);
-          frac = (uint32_t)Efx;
-          k = kx + 1;
+          A = A2;
+          away = (unsigned)(at + 16 * kBin) >= 32u * kBin;
+          n_chg += rn != r ? 1 : 0;
+          r = rn;
+          acc_cur |= 1u << e;
+          rb = lane > e ? r : rb;
         }
-        Efx = ((long long)bcur << 32) | frac;
+        frac = at & (kBin - 1);
+      } else if (path == kBlocks) {
+        // payload: bit 24 the move leaves the bin, bit 25 it touches a later one or may reach further than
+        // the next bin (looked up on its own), else the new fraction
+        constexpr uint32_t kRare = 0x03000000u;
+        uint32_t kc;
+        bool live = valid;
+        auto arm = [&]() {                 // after a bin change or a correction
+          pass();
+          const bool far = (unsigned)(dq + kBin) >= 2u * kBin;
+          kc = lane_key | (far || ((touched >> lane) & 1u) ? 0x02000000u : 0u);
+          if (far) {                       // a candidate wherever it lands
+            lo = (int)0x80000000u;
+            span = 0xffffffffu;
+          }
+          if (!live) span = 0u;
+        };
+        arm();
+        while (true) {
+          const int pos = frac + dq;
+          const uint32_t m = __reduce_min_sync(
+              kFullMask, (uint32_t)pos - (uint32_t)lo < span ? ((uint32_t)pos & 0x01ffffffu) | kc : kNoKey);
+          const int e = (int)(m >> 27);
+          if (m & kRare) {
+            if (m == kNoKey) break;        // every move left is rejected
+            const int pe = __shfl_sync(kFullMask, pos, e);
+            const int de = pe >> 24;
+            live = live && lane > e;
+            span = live ? span : 0u;
+            if (de != 0) {
+              if (!admits(e, de)) continue;
+              change_bin(e, de);
+            }
+            acc_cur |= 1u << e;
+            frac = pe & (kBin - 1);
+            if ((touched >> e) & 1u) push(e);
+            arm();
+          } else {
+            live = live && lane > e;
+            span = live ? span : 0u;
+            acc_cur |= 1u << e;
+            frac = (int)(m & 0xffffffu);
+          }
+        }
+      } else if (nvalid > 0) {
+        // Prefix sums S of the increments give every undecided move's position if all of them before it
+        // are accepted in the bin (which they are until one leaves the bin or meets an accepted move
+        // of this batch); sums wrap modulo 2^32, but up to the first exit they stay within 101 bins.
+        // payload: the increment of a rejected exit; kRare: an accepted one, one that may reach further
+        // than the next bin, or a move that meets an accepted one and takes its corrections when its turn
+        // comes (then every earlier move in `need` is an accepted one)
+        constexpr uint32_t kRare = 0x04000000u;
+        const uint32_t every = nvalid >= 32 ? 0xffffffffu : ((1u << nvalid) - 1u);
+        uint32_t need = sc | (uint32_t)tc.x | (uint32_t)tc.y | (uint32_t)tc.z | (uint32_t)tc.w;
+        uint32_t rej = 0u;                   // rejected moves
+        uint32_t S = valid ? (uint32_t)dq : 0u;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const uint32_t t = __shfl_up_sync(kFullMask, S, o);
+          if (lane >= o) S += t;
+        }
+        uint32_t base = (uint32_t)frac;
+        pass();
+        bool live = valid;
+        bool far;
+        uint32_t kc;
+        auto arm = [&]() {                   // after a correction
+          far = (unsigned)(dq + kBin) >= 2u * kBin;
+          kc = lane_key | ((uint32_t)dq & 0x03ffffffu);
+        };
+        arm();
+        while (true) {
+          const int pos = (int)(base + S);
+          const bool meet = need != 0u;
+          const uint32_t m = __reduce_min_sync(
+              kFullMask, live && (meet || (unsigned)pos >= (unsigned)kBin)
+                             ? kc | (meet || far || (uint32_t)pos - (uint32_t)lo < span ? kRare : 0u) : kNoKey);
+          const int e = (int)(m >> 27);
+          const uint32_t bit = 1u << e;
+          if (m & kRare) {
+            if (m == kNoKey) {               // the rest of the batch stays in the bin
+              frac = __shfl_sync(kFullMask, pos, nvalid - 1);
+              break;
+            }
+            uint32_t fix = __shfl_sync(kFullMask, need, e);
+            if (fix) {                       // move e takes its corrections
+              const float4 h0 = h4, d0 = d4;
+              const int dq0 = dq;
+              for (; fix; fix &= fix - 1u) {
+                const int j = __ffs(fix) - 1;
+                const uint32_t bj = 1u << j;
+                const float4 dj = C.ds[j];
+                const float J = coupling(tc, bj);
+                h4.x = fmaf(J, dj.x, h4.x);
+                h4.y = fmaf(J, dj.y, h4.y);
+                h4.z = fmaf(J, dj.z, h4.z);
+                if (lane == e && (sc & bj)) {
+                  replace(C.n[j]);
+                  same |= bj;
+                }
+              }
+              increment();
+              if (lane != e) {               // the others wait for their turn
+                h4 = h0;
+                d4 = d0;
+                dq = dq0;
+              } else {
+                need = 0u;
+              }
+              __syncwarp();
+              const int more = __shfl_sync(kFullMask, dq - dq0, e);
+              S += lane >= e ? (uint32_t)more : 0u;
+              arm();
+              continue;
+            }
+            const int pe = __shfl_sync(kFullMask, pos, e), de = __shfl_sync(kFullMask, dq, e);
+            live = live && lane > e;
+            if (admits(e, pe >> 24)) {
+              const int db = pe >> 24;
+              change_bin(e, db);
+              pass();
+              base -= (uint32_t)(db * kBin);
+            } else {
+              rej |= bit;
+              need &= ~bit;
+              base -= (uint32_t)de;
+            }
+          } else {
+            rej |= bit;
+            need &= ~bit;
+            live = live && lane > e;
+            base -= (uint32_t)((int)(m << 6) >> 6);
+          }
+        }
+        acc_cur = every & ~rej;
       }
-      // measured: blocks cost about 90 cycles per move whatever the rejected exits; the scan about
-      // 200 per batch plus 260 per event, so it wins below about 10 events per batch
+      // histogram: every move counts at the bin it leaves the walker in, i.e. the bin before the next move
+      if (!frozen && valid) atomicAdd(&H_s[lane == 0 ? r : rb], 1u);
+      n_rec += valid && ((uint32_t)hd.w & acc_cur) != 0u ? 1u : 0u;
+      pub_prev = acc_cur;
+      if ((uint32_t)all.y & acc_cur)       // moves superseded on their site by a later accepted one
+        pub_prev &= ~__reduce_or_sync(kFullMask, (acc_cur >> lane) & 1u ? same : 0u);
       if (nvalid > 0) {
         n_scan += path == kScan ? 1 : 0;
         n_blocks += path == kBlocks ? 1 : 0;
         n_seq += path == kSequential ? 1 : 0;
       }
-      path = forced >= 0 ? forced : ((n_rej + n_ev <= 10) ? kScan : (n_ev >= 6 ? kSequential : kBlocks));
-      // the batch's moves at the current bin
-      lng_seg += (long long)(nvalid - k_seg) * lnf_eff;
-      h_seg += hinc * (uint32_t)(nvalid - k_seg);
-      n_acc += __popc(acc_cur);
+      n_in = __popc(acc_cur);
+      n_exit = nvalid - n_in + n_chg;      // moves that left the bin, accepted or not
+      A += (long long)nvalid * lnf_eff;
+      n_acc += n_in;
       acc_prev = acc_cur;
-      pub_prev = acc_cur & ~sup;
+      acc_prev_rev = __brev(acc_cur);
     }
     // the last batch's spins
     if (nb > 0) {
-      publish(rec + ((nb - 1) & 1) * 32, pub_prev);
+      if ((pub_prev >> lane) & 1u)
+        lat.set_code(place_prev.x, make_float2(__int_as_float(place_prev.y), __int_as_float(place_prev.z)));
+      __syncwarp();
       named_arrive(kBarDone + ((nb - 1) & 1));
     }
+    const unsigned corrected = __reduce_add_sync(kFullMask, n_rec);
     if (lane == 0 && !bad) {
-      a.st.efx[slot] = Efx;
-      lng_s[bcur - wlo] = (Lng)lng_seg;
-      H_s[bcur - wlo] = h_seg;
+      a.st.efx[slot] = ((long long)(r + wlo) << 32) | (long long)(((uint32_t)frac << 8) | frac_low);
+      lng_s[r] = (Lng)A;
       a.st.steps[slot] = t0 + moves;
       a.st.accepts[slot] += n_acc;
-      a.st.recomputes[slot] += n_rec;
+      a.st.recomputes[slot] += corrected;
       a.st.path_batches[3 * (size_t)slot + 0] += n_scan;
       a.st.path_batches[3 * (size_t)slot + 1] += n_blocks;
       a.st.path_batches[3 * (size_t)slot + 2] += n_seq;
@@ -1045,8 +1054,7 @@ size_t walker_pipe_smem_bytes(bool traj, bool smem_lattice, int N, int W, int ow
   const size_t lng = align16((traj ? sizeof(double) : sizeof(long long)) * (size_t)W);
   const size_t h = align16((size_t)W * 4);
   const size_t real = traj ? sizeof(double) : sizeof(float);
-  const size_t recs = (traj ? sizeof(Rec<true>) : sizeof(Rec<false>)) * 64 + sizeof(int4) * 64;
-  size_t bytes = lng + h + 4 * kMaxSlotsPerSite + real * kMaxSlotsPerSite + recs + 8 * (size_t)own_entries;
+  size_t bytes = lng + h + 4 * kMaxSlotsPerSite + real * kMaxSlotsPerSite + batch_bytes(traj) + 8 * (size_t)own_entries;
   if (smem_lattice) bytes += smem_site_bytes(traj) * (size_t)N;
   return bytes;
 }
