@@ -15,7 +15,7 @@ BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "librewl.so")
 INCLUDE = os.path.join(os.path.dirname(HERE), "include")
 
-SOURCES = ["walker.cu", "walker_pipe.cu", "kernels.cu", "api.cu", "stitch_static.cu", "batch.cu", "mlp.cu"]
+SOURCES = ["walker.cu", "walker_pipe.cu", "energy.cu", "kernels.cu", "api.cu", "stitch_static.cu", "batch.cu", "mlp.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 NVCC_FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-ffp-contract=off",
               "-Xcompiler", "-O2", "--expt-relaxed-constexpr", "-I", INCLUDE, "-I", CSRC]

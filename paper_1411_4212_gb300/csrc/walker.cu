@@ -328,22 +328,15 @@ __global__ void __launch_bounds__(kWalkerThreads) walker_kernel(const WalkerArgs
       a.st.H[lbase + w] = H_s[w];
     }
   }
-  if (a.recompute && !a.init) {
+  // bcc production lattices: energy_update_kernel, after the walk
+  if (a.recompute && !a.init && (kTraj || a.geo.kind != 0)) {
     const double Ef = full_energy<kTraj>(a, off_s, lat, red, threadIdx.x, blockDim.x, 0);
     if (tid == 0) {
       if (kTraj) {
         const double d = fabs(Ef - a.st.E[slot]);
         if (d > a.st.drift[slot]) a.st.drift[slot] = d;
       } else {
-        const long long efx = a.st.efx[slot];
-        const double Er = a.win.e_min + a.win.dE * ((double)efx / kEnergyScale);
-        const double d = fabs(Ef - Er);
-        if (d > a.st.drift[slot]) a.st.drift[slot] = d;
-        long long nf = __double2ll_rn((Ef - a.win.e_min) / a.win.dE * kEnergyScale);
-        const long long lo_fx = (long long)wlo << 32;
-        const long long hi_fx = ((long long)(wlo + W) << 32) - 1;
-        nf = nf < lo_fx ? lo_fx : (nf > hi_fx ? hi_fx : nf);
-        a.st.efx[slot] = nf;
+        replace_energy(a, slot, wlo, Ef);
       }
     }
   }
@@ -418,8 +411,10 @@ cudaError_t launch_walkers(const WalkerArgs& a, int n_slots, bool traj, bool sme
     e = cudaFuncSetAttribute(walker_kernel<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e == cudaSuccess) walker_kernel<false, false><<<n_slots, kWalkerThreads, smem, stream>>>(a);
   }
-  if (e != cudaSuccess) return e;
-  return cudaGetLastError();
+  if (e == cudaSuccess) e = cudaGetLastError();
+  if (e == cudaSuccess && a.recompute && !a.init && !traj && a.geo.kind == 0)
+    e = launch_energy_update(a, n_slots, stream);
+  return e;
 }
 
 }  // namespace rewl

@@ -40,6 +40,12 @@ struct BatchLaunch {
 cudaError_t setup_walkers_batch(bool traj, int n_shells, int workers, size_t arena, int* blocks_per_sm);
 cudaError_t launch_walkers_batch(const BatchLaunch& b, cudaStream_t stream);
 
+// Full energy of every slot's configuration replaces the running energy (production, bcc), after the walk.
+cudaError_t launch_energy_update(const WalkerArgs& a, int n_slots, cudaStream_t stream);
+// The same over the (job, slot) items of a batch; walk_threads: threads per walker (the order of the sum).
+cudaError_t launch_energy_update_batch(const WalkerArgs* jobs, const int2* items, int n_items, int n_shells,
+                                       int walk_threads, cudaStream_t stream);
+
 struct ExchangeArgs {
   Windows win;
   WalkerState st;

@@ -22,6 +22,33 @@ struct Mode<false> {
   using Lng = long long;
 };
 
+struct ShellTable {
+  int dx[kMaxSlotsPerSite], dy[kMaxSlotsPerSite], dz[kMaxSlotsPerSite], sh[kMaxSlotsPerSite];
+  int z;
+};
+
+// Canonical bcc slot order: shell by shell (squared half-unit lengths 3, 4, 8, 11), lexicographic
+// (dx, dy, dz) inside a shell.
+constexpr ShellTable make_shells(int nsh) {
+  ShellTable t{};
+  constexpr int r2s[4] = {3, 4, 8, 11};
+  int z = 0;
+  for (int s = 0; s < nsh; ++s)
+    for (int a = -3; a <= 3; ++a)
+      for (int b = -3; b <= 3; ++b)
+        for (int c = -3; c <= 3; ++c) {
+          if (((a ^ b) & 1) != 0 || ((b ^ c) & 1) != 0) continue;
+          if (a * a + b * b + c * c != r2s[s]) continue;
+          t.dx[z] = a;
+          t.dy[z] = b;
+          t.dz[z] = c;
+          t.sh[z] = s;
+          ++z;
+        }
+  t.z = z;
+  return t;
+}
+
 // Spins of one configuration.
 // SpinPlanes: three FP64 arrays x[N], y[N], z[N] -- trajectory lattices, in global memory ([R][3][N])
 //   and in shared memory.
@@ -416,5 +443,18 @@ __device__ double full_energy(const WalkerArgs& a, const uint32_t* off_s, const 
   return -(double)a.geo.energy_weight * tot;
 }
 
+// Production: the recomputed energy Ef replaces the running energy of a slot (whose window starts at bin
+// wlo), kept inside the window; the difference counts as drift.  One thread.
+__device__ __forceinline__ void replace_energy(const WalkerArgs& a, int slot, int wlo, double Ef) {
+  const long long efx = a.st.efx[slot];
+  const double Er = a.win.e_min + a.win.dE * ((double)efx / kEnergyScale);
+  const double d = fabs(Ef - Er);
+  if (d > a.st.drift[slot]) a.st.drift[slot] = d;
+  long long nf = __double2ll_rn((Ef - a.win.e_min) / a.win.dE * kEnergyScale);
+  const long long lo_fx = (long long)wlo << 32;
+  const long long hi_fx = ((long long)(wlo + a.win.W) << 32) - 1;
+  nf = nf < lo_fx ? lo_fx : (nf > hi_fx ? hi_fx : nf);
+  a.st.efx[slot] = nf;
+}
 
 }  // namespace rewl

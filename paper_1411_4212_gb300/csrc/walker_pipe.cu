@@ -334,11 +334,12 @@ __device__ __forceinline__ void pipe_walk_slot(const WalkerArgs& a, const int sl
               ey = min(ey, 2 * L - ey);
               ez = min(ez, 2 * L - ez);
               const int r2 = ex * ex + ey * ey + ez * ez;
+              // (a shell without coupling changes nothing either)
               same |= r2 == 0 ? bit : 0u;
-              sh[0] |= r2 == 3 ? bit : 0u;
-              sh[1] |= NSH > 1 && r2 == 4 ? bit : 0u;
-              sh[2] |= NSH > 2 && r2 == 8 ? bit : 0u;
-              sh[3] |= NSH > 3 && r2 == 11 ? bit : 0u;
+              sh[0] |= r2 == 3 && Jsh[0] != Real(0) ? bit : 0u;
+              sh[1] |= NSH > 1 && r2 == 4 && Jsh[1] != Real(0) ? bit : 0u;
+              sh[2] |= NSH > 2 && r2 == 8 && Jsh[2] != Real(0) ? bit : 0u;
+              sh[3] |= NSH > 3 && r2 == 11 && Jsh[3] != Real(0) ? bit : 0u;
             }
           };
           sort_bits(m, ccur, scur, tcur);
@@ -784,7 +785,8 @@ __device__ __forceinline__ void pipe_walk_slot(const WalkerArgs& a, const int sl
         // of this batch); sums wrap modulo 2^32, but up to the first exit they stay within 101 bins.
         // payload: the increment of a rejected exit; kRare: an accepted one, one that may reach further
         // than the next bin, or a move that meets an accepted one and takes its corrections when its turn
-        // comes (then every earlier move in `need` is an accepted one)
+        // comes (then every earlier move in `need` is an accepted one); no increment beside kRare, so that
+        // no key of lane 31 is kNoKey
         constexpr uint32_t kRare = 0x04000000u;
         const uint32_t every = nvalid >= 32 ? 0xffffffffu : ((1u << nvalid) - 1u);
         uint32_t need = sc | (uint32_t)tc.x | (uint32_t)tc.y | (uint32_t)tc.z | (uint32_t)tc.w;
@@ -810,7 +812,7 @@ __device__ __forceinline__ void pipe_walk_slot(const WalkerArgs& a, const int sl
           const bool meet = need != 0u;
           const uint32_t m = __reduce_min_sync(
               kFullMask, live && (meet || (unsigned)pos >= (unsigned)kBin)
-                             ? kc | (meet || far || (uint32_t)pos - (uint32_t)lo < span ? kRare : 0u) : kNoKey);
+                             ? (meet || far || (uint32_t)pos - (uint32_t)lo < span ? lane_key | kRare : kc) : kNoKey);
           const int e = (int)(m >> 27);
           const uint32_t bit = 1u << e;
           if (m & kRare) {
