@@ -22,33 +22,6 @@
 
 namespace rewl {
 
-struct ShellTable {
-  int dx[kMaxSlotsPerSite], dy[kMaxSlotsPerSite], dz[kMaxSlotsPerSite], sh[kMaxSlotsPerSite];
-  int z;
-};
-
-// Canonical bcc slot order: shell by shell (squared half-unit lengths 3, 4, 8, 11), lexicographic
-// (dx, dy, dz) inside a shell.
-constexpr ShellTable make_shells(int nsh) {
-  ShellTable t{};
-  constexpr int r2s[4] = {3, 4, 8, 11};
-  int z = 0;
-  for (int s = 0; s < nsh; ++s)
-    for (int a = -3; a <= 3; ++a)
-      for (int b = -3; b <= 3; ++b)
-        for (int c = -3; c <= 3; ++c) {
-          if (((a ^ b) & 1) != 0 || ((b ^ c) & 1) != 0) continue;
-          if (a * a + b * b + c * c != r2s[s]) continue;
-          t.dx[z] = a;
-          t.dy[z] = b;
-          t.dz[z] = c;
-          t.sh[z] = s;
-          ++z;
-        }
-  t.z = z;
-  return t;
-}
-
 constexpr int kPairThreads = 64;   // resolver warp + producer warp
 constexpr int kWorkerThreads = 64;     // batched walker: threads per worker (one pair)
 
@@ -920,22 +893,12 @@ __device__ __forceinline__ void pipe_walk_slot(const WalkerArgs& a, const int sl
       a.st.lng_fx[lbase + w] = (long long)lng_s[w];
     a.st.H[lbase + w] = H_s[w];
   }
-  if (recompute) {
-    const double Ef = full_energy<kTraj>(a, off_s, lat, red, tid, nt, bar_sync);
-    if (tid == 0) {
-      if constexpr (kTraj) {
+  if constexpr (kTraj) {       // production: energy_update_kernel, after the walk
+    if (recompute) {
+      const double Ef = full_energy<kTraj>(a, off_s, lat, red, tid, nt, bar_sync);
+      if (tid == 0) {
         const double d = fabs(Ef - a.st.E[slot]);
         if (d > a.st.drift[slot]) a.st.drift[slot] = d;
-      } else {
-        const long long efx = a.st.efx[slot];
-        const double Er = a.win.e_min + a.win.dE * ((double)efx / kEnergyScale);
-        const double d = fabs(Ef - Er);
-        if (d > a.st.drift[slot]) a.st.drift[slot] = d;
-        long long nf = __double2ll_rn((Ef - a.win.e_min) / a.win.dE * kEnergyScale);
-        const long long lo_fx = (long long)wlo << 32;
-        const long long hi_fx = ((long long)(wlo + W) << 32) - 1;
-        nf = nf < lo_fx ? lo_fx : (nf > hi_fx ? hi_fx : nf);
-        a.st.efx[slot] = nf;
       }
     }
   }
@@ -1049,7 +1012,10 @@ cudaError_t launch_walkers_batch(const BatchLaunch& b, cudaStream_t stream) {
     default: return cudaErrorInvalidValue;
   }
 #undef REWL_BATCH_LAUNCH
-  return cudaGetLastError();
+  e = cudaGetLastError();
+  if (e == cudaSuccess && b.recompute && !b.traj)
+    e = launch_energy_update_batch(b.jobs, b.items, b.n_items, b.n_shells, kWorkerThreads, stream);
+  return e;
 }
 
 size_t walker_pipe_smem_bytes(bool traj, bool smem_lattice, int N, int W, int own_entries) {
@@ -1093,8 +1059,9 @@ static cudaError_t launch_pipe_shells(const WalkerArgs& a, const WalkerArgs* d_a
 cudaError_t launch_walkers_pipe(const WalkerArgs& a, const WalkerArgs* d_args, int n_slots, bool traj, size_t smem,
                                 cudaStream_t stream) {
   if (a.smem_lattice == (d_args != nullptr)) return cudaErrorInvalidValue;
-  return traj ? launch_pipe_shells<true>(a, d_args, n_slots, smem, stream)
-              : launch_pipe_shells<false>(a, d_args, n_slots, smem, stream);
+  if (traj) return launch_pipe_shells<true>(a, d_args, n_slots, smem, stream);
+  const cudaError_t e = launch_pipe_shells<false>(a, d_args, n_slots, smem, stream);
+  return e == cudaSuccess && a.recompute ? launch_energy_update(a, n_slots, stream) : e;
 }
 
 }  // namespace rewl
