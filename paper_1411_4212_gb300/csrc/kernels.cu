@@ -369,14 +369,6 @@ __device__ double warp_sum32_frag(const MergeArgs& a, size_t base, int n) {
   return p;
 }
 
-__device__ double warp_sum32(const double* x, int n) {
-  const int lane = threadIdx.x & 31;
-  double p = 0.0;
-  for (int i = lane; i < n; i += 32) p = __dadd_rn(p, x[i]);
-  for (int o = 16; o > 0; o >>= 1) p = __dadd_rn(p, __shfl_xor_sync(kFullMask, p, o));
-  return p;
-}
-
 // (1) per window k: A_k[w] = (sum_a (x_a[w] - mean_a)) / m, mean_a = sum32(x_a) / W.
 __global__ void merge_avg_kernel(const MergeArgs a) {
   extern __shared__ double means[];
@@ -395,79 +387,127 @@ __global__ void merge_avg_kernel(const MergeArgs a) {
   }
 }
 
-// (2)-(4) join points, shifts, assembly, mean removal.  One CTA.
-__global__ void merge_join_kernel(const MergeArgs a) {
-  extern __shared__ unsigned char js[];
-  double* shift = reinterpret_cast<double*>(js);
-  int* bst = reinterpret_cast<int*>(shift + a.h);
-  __shared__ double mean_s;
+// (2) per pair of windows (k, k+1), one warp: the interior overlap bin where the central-difference slopes of
+// the averages differ least (lowest bin on ties) into bstar[k], and the step of the shift there, A_k - A_{k+1},
+// into out[k] (out has at least h bins and is assembled afterwards).
+__global__ void merge_pairs_kernel(const MergeArgs a) {
+  const int lane = threadIdx.x & 31;
+  const int k = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  if (k + 1 >= a.h) return;
+  const int W = a.W;
+  const int sk = a.starts[k], sn = a.starts[k + 1];
+  const int lo = sn + 1, hi = sk + W - 2;
+  const double* Ak = a.avg + (size_t)k * W - sk;
+  const double* An = a.avg + (size_t)(k + 1) * W - sn;
+  double bv = __longlong_as_double(0x7ff0000000000000LL);
+  int bb = -1;
+  for (int b = lo + lane; b <= hi; b += 32) {
+    const double s1 = __dsub_rn(Ak[b + 1], Ak[b - 1]);
+    const double s2 = __dsub_rn(An[b + 1], An[b - 1]);
+    const double v = fabs(__dsub_rn(s1, s2));
+    if (v < bv) {              // lanes visit b in increasing order: first minimum kept
+      bv = v;
+      bb = b;
+    }
+  }
+  for (int o = 16; o > 0; o >>= 1) {
+    const double ov = __shfl_xor_sync(kFullMask, bv, o);
+    const int ob = __shfl_xor_sync(kFullMask, bb, o);
+    if (ob >= 0 && (bb < 0 || ov < bv || (ov == bv && ob < bb))) {
+      bv = ov;
+      bb = ob;
+    }
+  }
+  if (lane == 0) {
+    const int b = bb >= 0 ? bb : sn;
+    a.bstar[k] = b;
+    a.out[k] = __dsub_rn(Ak[b], An[b]);
+  }
+}
+
+// (3)-(4) shifts, assembly, mean removal.  One CTA; the assembled curve sits in shared memory when it fits (kSmem).
+// What bounds it: two chains of FP64 additions in the canonical order (62 cycles each): h shifts, and B / 32
+// terms per lane of the mean.  The search for a bin's window, one step after the other before, is a binary
+// search: bin b belongs to the first window k whose join bin lies above b, i.e. the first k whose running
+// maximum of join bins does.  Measured (300 windows, 16384 bins): 321 -> 57 us, the pairs above included.
+template <bool kSmem>
+__global__ void __launch_bounds__(1024) merge_join_kernel(const MergeArgs a) {
+  extern __shared__ __align__(16) unsigned char js[];
   const int h = a.h, W = a.W, B = a.B;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  const double inf = __longlong_as_double(0x7ff0000000000000LL);
-  for (int k = warp; k + 1 < h; k += nw) {
-    const int sk = a.starts[k], sn = a.starts[k + 1];
-    const int lo = sn + 1, hi = sk + W - 2;
-    const double* Ak = a.avg + (size_t)k * W;
-    const double* An = a.avg + (size_t)(k + 1) * W;
-    double bv = inf;
-    int bb = -1;
-    for (int b = lo + lane; b <= hi; b += 32) {
-      const double s1 = __dsub_rn(Ak[b + 1 - sk], Ak[b - 1 - sk]);
-      const double s2 = __dsub_rn(An[b + 1 - sn], An[b - 1 - sn]);
-      const double v = fabs(__dsub_rn(s1, s2));
-      if (v < bv) {            // lanes visit b in increasing order: first minimum kept
-        bv = v;
-        bb = b;
-      }
-    }
-    for (int o = 16; o > 0; o >>= 1) {
-      const double ov = __shfl_xor_sync(kFullMask, bv, o);
-      const int ob = __shfl_xor_sync(kFullMask, bb, o);
-      if (ob >= 0 && (bb < 0 || ov < bv || (ov == bv && ob < bb))) {
-        bv = ov;
-        bb = ob;
-      }
-    }
-    if (lane == 0) bst[k] = bb >= 0 ? bb : sn;
+  double* shift = reinterpret_cast<double*>(js);
+  double* curve = shift + h;
+  int* top = reinterpret_cast<int*>(curve + (kSmem ? B : 0));
+  int* start = top + h;
+  __shared__ double mean_s;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (int k = threadIdx.x; k < h; k += blockDim.x) {
+    shift[k] = k + 1 < h ? a.out[k] : 0.0;
+    start[k] = a.starts[k];
   }
   __syncthreads();
   if (threadIdx.x == 0) {
-    shift[0] = 0.0;
-    for (int k = 0; k + 1 < h; ++k) {
-      const int b = bst[k];
-      shift[k + 1] = __dadd_rn(shift[k], __dsub_rn(a.avg[(size_t)k * W + (b - a.starts[k])],
-                                                   a.avg[(size_t)(k + 1) * W + (b - a.starts[k + 1])]));
+    double t = 0.0;
+#pragma unroll 8
+    for (int k = 0; k < h; ++k) {
+      const double step = shift[k];
+      shift[k] = t;
+      t = __dadd_rn(t, step);
+    }
+  } else if (warp == 1) {      // running maximum of the join bins
+    int before = -1;
+    for (int k0 = 0; k0 + 1 < h; k0 += 32) {
+      int v = k0 + lane + 1 < h ? a.bstar[k0 + lane] : -1;
+      for (int o = 1; o < 32; o <<= 1) {
+        const int u = __shfl_up_sync(kFullMask, v, o);
+        if (lane >= o) v = max(v, u);
+      }
+      v = max(v, before);
+      if (k0 + lane + 1 < h) top[k0 + lane] = v;
+      before = __shfl_sync(kFullMask, v, 31);
     }
   }
   __syncthreads();
+  double* y = kSmem ? curve : a.out;
   for (int b = threadIdx.x; b < B; b += blockDim.x) {
-    int k = 0;
-    while (k + 1 < h && b >= bst[k]) ++k;
-    a.out[b] = __dadd_rn(a.avg[(size_t)k * W + (b - a.starts[k])], shift[k]);
+    int lo = 0, hi = h - 1;                // first k with top[k] > b, h - 1 if none
+    while (lo < hi) {
+      const int mid = (lo + hi) >> 1;
+      if (top[mid] > b)
+        hi = mid;
+      else
+        lo = mid + 1;
+    }
+    y[b] = __dadd_rn(a.avg[(size_t)lo * W + (b - start[lo])], shift[lo]);
   }
   __syncthreads();
   if (warp == 0) {
-    const double s = warp_sum32(a.out, B);
-    if (lane == 0) mean_s = __ddiv_rn(s, (double)B);
+    double p = 0.0;
+#pragma unroll 8
+    for (int i = lane; i < B; i += 32) p = __dadd_rn(p, y[i]);
+    for (int o = 16; o > 0; o >>= 1) p = __dadd_rn(p, __shfl_xor_sync(kFullMask, p, o));
+    if (lane == 0) mean_s = __ddiv_rn(p, (double)B);
   }
   __syncthreads();
   const double mu = mean_s;
-  for (int b = threadIdx.x; b < B; b += blockDim.x) a.out[b] = __dsub_rn(a.out[b], mu);
-  if (a.bstar)
-    for (int k = threadIdx.x; k + 1 < h; k += blockDim.x) a.bstar[k] = bst[k];
+  for (int b = threadIdx.x; b < B; b += blockDim.x) a.out[b] = __dsub_rn(y[b], mu);
 }
 
 cudaError_t launch_merge(const MergeArgs& a, cudaStream_t stream) {
   merge_avg_kernel<<<a.h, 256, sizeof(double) * (size_t)a.m, stream>>>(a);
+  if (a.h > 1) merge_pairs_kernel<<<(a.h + 2) / 4, 128, 0, stream>>>(a);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  const size_t js = sizeof(double) * (size_t)a.h + sizeof(int) * (size_t)a.h;
-  if (js > 48 * 1024) {
-    e = cudaFuncSetAttribute(merge_join_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)js);
-    if (e != cudaSuccess) return e;
+  const size_t js = (sizeof(double) + 2 * sizeof(int)) * (size_t)a.h;
+  const size_t with_curve = js + sizeof(double) * (size_t)a.B;
+  if (with_curve <= 200 * 1024) {          // up to about 25000 bins
+    e = cudaFuncSetAttribute(merge_join_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+    if (e == cudaSuccess) merge_join_kernel<true><<<1, 1024, with_curve, stream>>>(a);
+  } else {
+    if (js > 48 * 1024)
+      e = cudaFuncSetAttribute(merge_join_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)js);
+    if (e == cudaSuccess) merge_join_kernel<false><<<1, 1024, js, stream>>>(a);
   }
-  merge_join_kernel<<<1, 1024, js, stream>>>(a);
-  return cudaGetLastError();
+  return e == cudaSuccess ? cudaGetLastError() : e;
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -475,19 +515,13 @@ cudaError_t launch_merge(const MergeArgs& a, cudaStream_t stream) {
 // var = sum w (E - U)^2 / Z (two passes), C/N = var / (N T^2), ln Z = max + ln(sum w).
 // One CTA per temperature.
 // ------------------------------------------------------------------------------------------------
-__device__ double block_reduce(double v, double* red, bool is_max) {
-  for (int o = 16; o > 0; o >>= 1) {
-    const double ov = __shfl_xor_sync(kFullMask, v, o);
-    v = is_max ? fmax(v, ov) : v + ov;
-  }
+__device__ double block_sum(double v, double* red) {
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(kFullMask, v, o);
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
   __syncthreads();
   if (threadIdx.x < 32) {
-    double x = threadIdx.x < (blockDim.x >> 5) ? red[threadIdx.x] : (is_max ? -1e308 : 0.0);
-    for (int o = 16; o > 0; o >>= 1) {
-      const double ox = __shfl_xor_sync(kFullMask, x, o);
-      x = is_max ? fmax(x, ox) : x + ox;
-    }
+    double x = threadIdx.x < (blockDim.x >> 5) ? red[threadIdx.x] : 0.0;
+    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(kFullMask, x, o);
     if (threadIdx.x == 0) red[32] = x;
   }
   __syncthreads();
@@ -496,30 +530,129 @@ __device__ double block_reduce(double v, double* red, bool is_max) {
   return r;
 }
 
-__global__ void thermo_kernel(const double* lng, const double* E, int B, double n_spins, const double* T,
-                              double* U, double* C, double* lnZ) {
+// FP64 numbers as signed integers in the same order (NaN at the ends by its sign), and back.
+__device__ __forceinline__ long long order_key(double v) {
+  const long long b = __double_as_longlong(v);
+  return b ^ ((b >> 63) & 0x7fffffffffffffffLL);
+}
+__device__ __forceinline__ double order_value(long long k) {
+  return __longlong_as_double(k ^ ((k >> 63) & 0x7fffffffffffffffLL));
+}
+
+// e^x for x <= 0 (0 below -708, NaN for NaN) in integer arithmetic, within about a unit in the last place:
+// this GPU issues less than two FP64 operations per clock and SM, but 64-bit products of integers at a tenth
+// of its FP32 rate.  -x log2(e) = n + j/64 + r in 2^-53 units, r < 1/64;  e^x = 2^-n 2^(-j/64) 2^-r with the
+// middle factor from a table (2^-63 units) and the last by its Taylor polynomial of degree 6 (error 3e-18).
+constexpr int kPow2 = 64;
+__device__ __forceinline__ double exp_fixed(double x, const unsigned long long* pow2) {
+  const unsigned long long bits = (unsigned long long)__double_as_longlong(x) & 0x7fffffffffffffffULL;
+  if (bits >= 0x4086200000000000ULL) return bits > 0x7ff0000000000000ULL ? x : 0.0;   // |x| >= 708
+  const int e = (int)(bits >> 52) - 1023;
+  const unsigned long long m = (bits & 0xfffffffffffffULL) | 0x10000000000000ULL;
+  // |x| in 2^-54 units (e <= 9); below 2^-54 nothing is left of it
+  const unsigned long long q = e >= -2 ? m << (e + 2) : (e >= -54 ? m >> (-2 - e) : 0ULL);
+  const unsigned long long t = __umul64hi(q, 0xb8aa3b295c17f0bcULL);     // log2(e) in 2^-63 units
+  const unsigned long long u = (t << 17) >> 6;                            // r in 2^-64 units
+  unsigned long long v = 0x00050c244be1b1e2ULL;                            // (ln 2)^i / i! in 2^-63 units, i = 6 .. 0
+  v = 0x002bb0ffcf14ce62ULL - __umul64hi(u, v);
+  v = 0x013b2ab6fba4e773ULL - __umul64hi(u, v);
+  v = 0x071ac235c1282fe3ULL - __umul64hi(u, v);
+  v = 0x1ebfbdff82c58ea8ULL - __umul64hi(u, v);
+  v = 0x58b90bfbe8e7bcd6ULL - __umul64hi(u, v);
+  v = 0x8000000000000000ULL - __umul64hi(u, v);
+  const unsigned long long w = __umul64hi(pow2[(t >> 47) & 63], v);        // (1/2, 1] in 2^-62 units
+  // rounded to 53 bits; a carry into the next power of two is right as it stands
+  return __longlong_as_double((long long)(((1021ULL - (t >> 53)) << 52) + ((w + 256) >> 9)));
+}
+
+// 2^(-j/64) in 2^-63 units, from the six factors 2^(-1/2) .. 2^(-1/64) in 2^-64 units.
+__device__ __forceinline__ unsigned long long pow2_entry(int j) {
+  const unsigned long long f[6] = {0xb504f333f9de6484ULL, 0xd744fccad69d6af4ULL,
+                                 0xeac0c6e7dd24392fULL, 0xf5257d152486cc2cULL,
+                                 0xfa83b2db722a033aULL, 0xfd3e0c0cf486c175ULL};
+  unsigned long long v = 0x8000000000000000ULL;
+#pragma unroll
+  for (int i = 0; i < 6; ++i)
+    if ((j >> (5 - i)) & 1) v = __umul64hi(v, f[i]);
+  return v;
+}
+
+// kCached: at most kThermoKept bins per thread, whose weights stay in registers between the passes.
+// What bounds it: FP64 issue.  Per bin and temperature seven FP64 operations are left (of 46 with the library's
+// exponential in both passes and FP64 maxima).  Measured: 281 temperatures x 16384 bins 451 -> 99 us.
+constexpr int kThermoKept = 16;
+template <bool kCached>
+__global__ void __launch_bounds__(1024) thermo_kernel(const double* __restrict__ lng, const double* __restrict__ E,
+                                                      int B, double n_spins, const double* __restrict__ T, double* U,
+                                                      double* C, double* lnZ) {
   __shared__ double red[33];
+  __shared__ long long red_key[33];
+  __shared__ unsigned long long pow2[kPow2];
   const double t = T[blockIdx.x];
   const double beta = 1.0 / t;
-  double mx = -1e308;
-  for (int b = threadIdx.x; b < B; b += blockDim.x) mx = fmax(mx, lng[b] - E[b] * beta);
-  mx = block_reduce(mx, red, true);
-  double z = 0.0, e1 = 0.0;
-  for (int b = threadIdx.x; b < B; b += blockDim.x) {
-    const double w = exp(lng[b] - E[b] * beta - mx);
-    z += w;
-    e1 += w * E[b];
+  if (threadIdx.x < kPow2) pow2[threadIdx.x] = pow2_entry(threadIdx.x);
+  double x[kThermoKept];
+  // the largest exponent
+  long long key = order_key(-1e308);
+  if constexpr (kCached) {
+#pragma unroll
+    for (int i = 0; i < kThermoKept; ++i) {
+      const int b = threadIdx.x + i * (int)blockDim.x;
+      x[i] = b < B ? fma(-E[b], beta, lng[b]) : -1e308;
+      key = max(key, order_key(x[i]));
+    }
+  } else {
+    for (int b = threadIdx.x; b < B; b += blockDim.x) key = max(key, order_key(fma(-E[b], beta, lng[b])));
   }
-  z = block_reduce(z, red, false);
-  e1 = block_reduce(e1, red, false);
+  for (int o = 16; o > 0; o >>= 1) key = max(key, (long long)__shfl_xor_sync(kFullMask, key, o));
+  if ((threadIdx.x & 31) == 0) red_key[threadIdx.x >> 5] = key;
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    key = threadIdx.x < (blockDim.x >> 5) ? red_key[threadIdx.x] : order_key(-1e308);
+    for (int o = 16; o > 0; o >>= 1) key = max(key, (long long)__shfl_xor_sync(kFullMask, key, o));
+    if (threadIdx.x == 0) red_key[32] = key;
+  }
+  __syncthreads();
+  const double mx = order_value(red_key[32]);
+  double z = 0.0, e1 = 0.0;
+  if constexpr (kCached) {
+#pragma unroll
+    for (int i = 0; i < kThermoKept; ++i) {
+      const int b = threadIdx.x + i * (int)blockDim.x;
+      if (b < B) {
+        x[i] = exp_fixed(x[i] - mx, pow2);
+        z += x[i];
+        e1 = fma(x[i], E[b], e1);
+      }
+    }
+  } else {
+    for (int b = threadIdx.x; b < B; b += blockDim.x) {
+      const double w = exp_fixed(fma(-E[b], beta, lng[b]) - mx, pow2);
+      z += w;
+      e1 = fma(w, E[b], e1);
+    }
+  }
+  z = block_sum(z, red);
+  e1 = block_sum(e1, red);
   const double u = e1 / z;
   double v = 0.0;
-  for (int b = threadIdx.x; b < B; b += blockDim.x) {
-    const double w = exp(lng[b] - E[b] * beta - mx);
-    const double d = E[b] - u;
-    v += w * d * d;
+  if constexpr (kCached) {
+#pragma unroll
+    for (int i = 0; i < kThermoKept; ++i) {
+      const int b = threadIdx.x + i * (int)blockDim.x;
+      if (b < B) {
+        const double d = E[b] - u;
+        v = fma(x[i] * d, d, v);
+      }
+    }
+  } else {
+    for (int b = threadIdx.x; b < B; b += blockDim.x) {
+      const double w = exp_fixed(fma(-E[b], beta, lng[b]) - mx, pow2);
+      const double d = E[b] - u;
+      v = fma(w * d, d, v);
+    }
   }
-  v = block_reduce(v, red, false) / z;
+  v = block_sum(v, red) / z;
   if (threadIdx.x == 0) {
     if (U) U[blockIdx.x] = u;
     if (C) C[blockIdx.x] = v * beta * beta / n_spins;
@@ -529,7 +662,12 @@ __global__ void thermo_kernel(const double* lng, const double* E, int B, double 
 
 cudaError_t launch_thermo(const double* lng, const double* E, int B, double n_spins, const double* T, int nT,
                           double* U, double* C, double* lnZ, cudaStream_t stream) {
-  thermo_kernel<<<nT, 256, 0, stream>>>(lng, E, B, n_spins, T, U, C, lnZ);
+  if (B <= 256 * kThermoKept)
+    thermo_kernel<true><<<nT, 256, 0, stream>>>(lng, E, B, n_spins, T, U, C, lnZ);
+  else if (B <= 1024 * kThermoKept)
+    thermo_kernel<true><<<nT, 1024, 0, stream>>>(lng, E, B, n_spins, T, U, C, lnZ);
+  else
+    thermo_kernel<false><<<nT, 1024, 0, stream>>>(lng, E, B, n_spins, T, U, C, lnZ);
   return cudaGetLastError();
 }
 
