@@ -6,6 +6,7 @@
 #include <chrono>
 #include <cmath>
 #include <cstring>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -94,7 +95,9 @@ struct rewl_handle {
   double* d_avg = nullptr;
   int32_t* d_bstar = nullptr;
   double* d_merge = nullptr;
-  std::vector<void*> allocations;
+  unsigned char* arena = nullptr;   // every array above, one allocation
+  size_t walkers_bytes = 0;         // its first part: ln g, H, and from small_begin on the per-slot arrays
+  size_t small_begin = 0;
 
   bool initialized = false;
   bool broken = false;
@@ -103,6 +106,73 @@ struct rewl_handle {
   unsigned long long prev_ex_att = 0, prev_ex_acc = 0;
   std::string err;
 };
+
+// ---- device memory of the library ------------------------------------------------------------------
+// One stream-ordered memory pool per device, created by the first call that needs it, apart from the
+// device's default pool (whose settings belong to the host program).  A fresh cudaMalloc, or an allocation
+// from a pool that has given everything back, costs 50 to 300 us on GB300; a run's handle needs some 25
+// arrays, and thermodynamics, joining and the network's calls need scratch every time.  The pool keeps at
+// most 64 MiB that is not in use, and 4 MiB once the last handle and model are gone.  It is safe with several
+// threads and streams: the driver orders a block's next use after its last.
+namespace {
+
+constexpr int kMaxDevices = 128;
+constexpr unsigned long long kPoolKept = 64ull << 20, kPoolIdle = 4ull << 20;
+std::mutex g_pool_mu;
+cudaMemPool_t g_pool[kMaxDevices] = {};
+long long g_pool_users = 0;
+
+cudaError_t device_pool(cudaMemPool_t* pool) {
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
+  std::lock_guard<std::mutex> lock(g_pool_mu);
+  if (!g_pool[dev]) {
+    cudaMemPoolProps props{};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.handleTypes = cudaMemHandleTypeNone;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = dev;
+    cudaMemPool_t p = nullptr;
+    e = cudaMemPoolCreate(&p, &props);
+    if (e != cudaSuccess) return e;
+    unsigned long long kept = kPoolKept;
+    e = cudaMemPoolSetAttribute(p, cudaMemPoolAttrReleaseThreshold, &kept);
+    if (e != cudaSuccess) {
+      cudaMemPoolDestroy(p);
+      return e;
+    }
+    g_pool[dev] = p;
+  }
+  *pool = g_pool[dev];
+  return cudaSuccess;
+}
+
+}  // namespace
+
+cudaError_t rewl::pool_alloc(void** p, size_t bytes, cudaStream_t stream) {
+  *p = nullptr;
+  cudaMemPool_t pool = nullptr;
+  const cudaError_t e = device_pool(&pool);
+  return e == cudaSuccess ? cudaMallocFromPoolAsync(p, std::max<size_t>(bytes, 1), pool, stream) : e;
+}
+
+void rewl::pool_free(void* p, cudaStream_t stream) {
+  if (p) cudaFreeAsync(p, stream);
+}
+
+void rewl::pool_retain() {
+  std::lock_guard<std::mutex> lock(g_pool_mu);
+  ++g_pool_users;
+}
+
+void rewl::pool_release() {
+  std::lock_guard<std::mutex> lock(g_pool_mu);
+  if (--g_pool_users > 0) return;
+  for (cudaMemPool_t p : g_pool)
+    if (p) cudaMemPoolTrimTo(p, kPoolIdle);
+}
 
 namespace {
 
@@ -124,16 +194,6 @@ rewl_status fail(rewl_handle* h, rewl_status s, const std::string& msg) {
     if (e_ != cudaSuccess)                                                                      \
       return fail((h), REWL_ECUDA, std::string(#call) + ": " + cudaGetErrorString(e_));         \
   } while (0)
-
-template <class T>
-rewl_status dev_alloc(rewl_handle* h, T** p, size_t count) {
-  void* q = nullptr;
-  cudaError_t e = cudaMalloc(&q, std::max<size_t>(count, 1) * sizeof(T));
-  if (e != cudaSuccess) return fail(h, REWL_ENOMEM, std::string("cudaMalloc: ") + cudaGetErrorString(e));
-  h->allocations.push_back(q);
-  *p = static_cast<T*>(q);
-  return REWL_OK;
-}
 
 // bcc offsets in half lattice units, shell by shell (squared lengths 3, 4, 8, 11), lexicographic
 // (dx, dy, dz) inside a shell.  This is the slot order of the local-field sum.
@@ -158,13 +218,19 @@ int bcc_offsets(int n_shells, std::vector<std::array<int, 3>>& off, std::vector<
 double lt_ground_state(int L, const std::vector<std::array<int, 3>>& off, const std::vector<double>& Jslot) {
   const double pi = 3.14159265358979323846;
   double best = -INFINITY;
+  // the phases are whole multiples of pi / L: their cosines, once each
+  int reach = 0;
+  for (const auto& d : off) reach = std::max(reach, std::abs(d[0]) + std::abs(d[1]) + std::abs(d[2]));
+  reach *= 2 * L - 1;
+  std::vector<double> cosine(2 * (size_t)reach + 1);
+  for (int dot = -reach; dot <= reach; ++dot) cosine[dot + reach] = std::cos(pi * (double)dot / (double)L);
   for (int n1 = 0; n1 < 2 * L; ++n1)
     for (int n2 = 0; n2 < 2 * L; ++n2)
       for (int n3 = 0; n3 < 2 * L; ++n3) {
         double jq = 0.0;
         for (size_t j = 0; j < off.size(); ++j) {
           const int dot = n1 * off[j][0] + n2 * off[j][1] + n3 * off[j][2];
-          jq = jq + Jslot[j] * std::cos(pi * (double)dot / (double)L);
+          jq = jq + Jslot[j] * cosine[dot + reach];
         }
         if (jq > best) best = jq;
       }
@@ -305,6 +371,25 @@ rewl_status check_whole(rewl_handle* h) {
   return REWL_OK;
 }
 
+// Host copy of the first part of a handle's arena: the small per-slot arrays and exchange counters, and with
+// `tables` ln g and H before them.  One copy; at(d) is where array d is found.
+struct Walkers {
+  std::vector<unsigned char> buf;
+  const unsigned char* from = nullptr;
+  rewl_status read(rewl_handle* h, bool tables) {
+    const size_t begin = tables ? 0 : h->small_begin;
+    from = h->arena + begin;
+    buf.resize(h->walkers_bytes - begin);
+    CUDA_TRY(h, cudaMemcpyAsync(buf.data(), from, buf.size(), cudaMemcpyDeviceToHost, h->stream));
+    CUDA_TRY(h, cudaStreamSynchronize(h->stream));
+    return REWL_OK;
+  }
+  template <class T>
+  const T* at(const T* d) const {
+    return reinterpret_cast<const T*>(buf.data() + (reinterpret_cast<const unsigned char*>(d) - from));
+  }
+};
+
 }  // namespace
 
 void rewl::set_handleless_error(const std::string& msg) { g_last_error = msg; }
@@ -318,8 +403,12 @@ const char* rewl_last_error(const rewl_handle* h) {
 
 void rewl_destroy(rewl_handle* h) {
   if (!h) return;
-  if (h->stream) cudaStreamSynchronize(h->stream);
-  for (void* p : h->allocations) cudaFree(p);
+  if (h->arena) {
+    // the handle's stream has waited for every batch that used the arrays
+    cudaStreamSynchronize(h->stream);
+    pool_free(h->arena, nullptr);
+  }
+  pool_release();
   delete h;
 }
 
@@ -332,6 +421,7 @@ static rewl_status create_impl(const rewl_lattice* lat, const rewl_couplings* cp
   *out = nullptr;
   if (!lat || !cpl || !win || !cfg) return fail(nullptr, REWL_EINVAL, "NULL argument");
   auto* h = new rewl_handle();
+  pool_retain();
   auto bad = [&](const std::string& msg) {
     g_last_error = msg;
     rewl_destroy(h);
@@ -414,12 +504,9 @@ static rewl_status create_impl(const rewl_lattice* lat, const rewl_couplings* cp
     g.energy_weight = 1.0f;
     // E0 = -1/2 sum_i sum_j J_ij for the aligned state, site by site in slot order (production
     // uses the FP32 couplings its energy changes are computed with)
-    double acc = 0.0;
-    for (int i = 0; i < h->N; ++i) {
-      double row = 0.0;
-      for (int j = 0; j < z; ++j) row = row + (h->traj ? Jslot[j] : (double)(float)Jslot[j]);
-      acc = acc + row;
-    }
+    double acc = 0.0, row = 0.0;
+    for (int j = 0; j < z; ++j) row = row + (h->traj ? Jslot[j] : (double)(float)Jslot[j]);
+    for (int i = 0; i < h->N; ++i) acc = acc + row;
     h->E0 = -0.5 * acc;
     if (std::isnan(win->e_min) || std::isnan(win->e_max)) {
       h->e_min = lt_ground_state(h->L, off, Jslot);
@@ -572,49 +659,46 @@ static rewl_status create_impl(const rewl_lattice* lat, const rewl_couplings* cp
     h->pipe = h->pipe_smem_bytes + 1024 <= (size_t)max_smem;
   }
 
-  const size_t S = h->S, W = h->W, N = h->N;
-  rewl_status st = REWL_OK;
-  auto A = [&](auto** p, size_t count) {
-    if (st == REWL_OK) st = dev_alloc(h, p, count);
-  };
+  const size_t S = h->S, W = h->W, N = h->N, X = (size_t)std::max(h->h - 1, 1);
   // spins: FP64 planes [S][3][N] (trajectory) or octahedral FP32 codes [S][N] float2 (production)
   const size_t spin_bytes = h->traj ? S * 3 * N * sizeof(double) : S * N * sizeof(float2);
-  void** spins_pp = &h->d_spins;
-  {
-    unsigned char* sp = nullptr;
-    A(&sp, spin_bytes);
-    *spins_pp = sp;
-  }
-  A(&h->d_perm, S);
-  A(&h->d_H, S * W);
-  if (h->traj) {
+  // One allocation for every array, 256-byte aligned.  First what the read-backs want (ln g and H, then the
+  // small per-slot arrays, so that each is one copy), then the rest.
+  std::vector<std::pair<void**, size_t>> parts;
+  auto A = [&](auto** p, size_t count) {
+    parts.emplace_back(reinterpret_cast<void**>(p), (std::max<size_t>(count, 1) * sizeof(**p) + 255) & ~(size_t)255);
+  };
+  if (h->traj)
     A(&h->d_lng, S * W);
+  else
+    A(&h->d_lng_fx, S * W);
+  A(&h->d_H, S * W);
+  const size_t n_tables = parts.size();
+  if (h->traj) {
     A(&h->d_E, S);
     A(&h->d_bin, S);
   } else {
-    A(&h->d_lng_fx, S * W);
     A(&h->d_efx, S);
     A(&h->d_lnf_fx, S);
   }
   A(&h->d_lnf, S);
+  A(&h->d_perm, S);
   A(&h->d_stage, S);
   A(&h->d_steps, S);
   A(&h->d_accepts, S);
-  A(&h->d_recomputes, S);
-  A(&h->d_path_batches, 3 * S);
   A(&h->d_init_moves, S);
   A(&h->d_drift, S);
+  A(&h->d_ex_att, X);
+  A(&h->d_ex_acc, X);
+  const size_t n_walkers = parts.size();
+  A(&h->d_recomputes, S);
+  A(&h->d_path_batches, 3 * S);
   A(&h->d_ctrl, 4);
   A(&h->d_wargs, 1);
   A(&h->d_ex_index, 1);
   A(&h->d_rt_last, S);
   A(&h->d_rt_count, S);
-  A(&h->d_ex_att, std::max(h->h - 1, 1));
-  A(&h->d_ex_acc, std::max(h->h - 1, 1));
   A(&h->d_starts, h->h);
-  A(&h->d_avg, (size_t)h->h * W);
-  A(&h->d_bstar, std::max(h->h - 1, 1));
-  A(&h->d_merge, h->B);
   if (h->part) {
     A(&h->d_gid, S);
     A(&h->d_pos_of, h->S_global);
@@ -627,78 +711,74 @@ static rewl_status create_impl(const rewl_lattice* lat, const rewl_couplings* cp
     A(&h->d_tab_Jf, (size_t)h->z * N);
     A(&h->d_tab_Jd, (size_t)h->z * N);
   }
-  if (st != REWL_OK) {
+  unsigned char* spins = nullptr;
+  A(&spins, spin_bytes);
+  const size_t n_zeroed = parts.size();    // everything up to here starts as zeros
+  A(&h->d_avg, (size_t)h->h * W);
+  A(&h->d_bstar, X);
+  A(&h->d_merge, h->B);
+  std::vector<size_t> at(parts.size() + 1, 0);
+  for (size_t i = 0; i < parts.size(); ++i) at[i + 1] = at[i] + parts[i].second;
+  void* arena = nullptr;
+  ce = pool_alloc(&arena, at.back(), h->stream);
+  if (ce != cudaSuccess) {
+    g_last_error = std::string("device memory: ") + cudaGetErrorString(ce);
     rewl_destroy(h);
-    return st;
+    return REWL_ENOMEM;
   }
+  h->arena = static_cast<unsigned char*>(arena);
+  for (size_t i = 0; i < parts.size(); ++i) *parts[i].first = h->arena + at[i];
+  h->d_spins = spins;
+  h->small_begin = at[n_tables];
+  h->walkers_bytes = at[n_walkers];
   g.tab_nbr = h->d_tab_nbr;
   g.tab_Jf = h->d_tab_Jf;
   g.tab_Jd = h->d_tab_Jd;
 
-  // ---- initial state: every configuration aligned along +z ----
+  // ---- initial state: every configuration aligned along +z (FP64 planes with z = 1, or the code (0, 0)) ----
+  ce = cudaMemsetAsync(h->arena, 0, at[n_zeroed], h->stream);
   auto up = [&](void* d, const void* src, size_t bytes) {
-    if (ce == cudaSuccess) ce = cudaMemcpy(d, src, bytes, cudaMemcpyHostToDevice);
+    if (ce == cudaSuccess) ce = cudaMemcpyAsync(d, src, bytes, cudaMemcpyHostToDevice, h->stream);
   };
-  auto zero = [&](void* d, size_t bytes) {
-    if (ce == cudaSuccess) ce = cudaMemset(d, 0, bytes);
-  };
-  // every configuration starts aligned along +z: FP64 planes with z = 1, or the code (0, 0)
   if (h->traj) {
     std::vector<unsigned char> sp(spin_bytes, 0);
     const double one = 1.0;
     for (size_t r = 0; r < S; ++r)
       for (size_t i = 0; i < N; ++i) std::memcpy(sp.data() + (r * 3 * N + 2 * N + i) * sizeof(double), &one, sizeof one);
     up(h->d_spins, sp.data(), sp.size());
-  } else {
-    zero(h->d_spins, spin_bytes);
+    if (ce == cudaSuccess) ce = cudaStreamSynchronize(h->stream);
   }
-  std::vector<int32_t> perm(S);
-  for (size_t s = 0; s < S; ++s) perm[s] = (int32_t)s;
-  up(h->d_perm, perm.data(), S * sizeof(int32_t));
-  zero(h->d_H, S * W * sizeof(uint32_t));
-  std::vector<double> lnf(S, h->lnf_initial);
-  up(h->d_lnf, lnf.data(), S * sizeof(double));
-  if (h->traj) {
-    zero(h->d_lng, S * W * sizeof(double));
-    std::vector<double> E(S, h->E0);
-    std::vector<int32_t> b(S, bin_of(h->E0, h->e_min, h->dE));
-    up(h->d_E, E.data(), S * sizeof(double));
-    up(h->d_bin, b.data(), S * sizeof(int32_t));
-  } else {
-    zero(h->d_lng_fx, S * W * sizeof(long long));
-    std::vector<long long> efx(S, std::llrint((h->E0 - h->e_min) / h->dE * kEnergyScale));
-    std::vector<long long> lf(S, std::llrint(h->lnf_initial * kLngScale));
-    up(h->d_efx, efx.data(), S * sizeof(long long));
-    up(h->d_lnf_fx, lf.data(), S * sizeof(long long));
-    for (auto& v : lnf) v = (double)lf[0] * kLngUnit;
-    up(h->d_lnf, lnf.data(), S * sizeof(double));
+  // the small per-slot arrays as one block
+  std::vector<unsigned char> block(at[n_walkers] - at[n_tables], 0);
+  auto host = [&](auto* d) { return reinterpret_cast<decltype(d)>(block.data() + (reinterpret_cast<unsigned char*>(d) - (h->arena + h->small_begin))); };
+  std::vector<float> jf(h->tab_J.size());
+  const long long lf = std::llrint(h->lnf_initial * kLngScale);
+  for (size_t s = 0; s < S; ++s) {
+    host(h->d_perm)[s] = (int32_t)s;
+    if (h->traj) {
+      host(h->d_lnf)[s] = h->lnf_initial;
+      host(h->d_E)[s] = h->E0;
+      host(h->d_bin)[s] = bin_of(h->E0, h->e_min, h->dE);
+    } else {
+      host(h->d_efx)[s] = std::llrint((h->E0 - h->e_min) / h->dE * kEnergyScale);
+      host(h->d_lnf_fx)[s] = lf;
+      host(h->d_lnf)[s] = (double)lf * kLngUnit;
+    }
   }
-  zero(h->d_stage, S * sizeof(int32_t));
-  zero(h->d_steps, S * sizeof(long long));
-  zero(h->d_accepts, S * sizeof(long long));
-  zero(h->d_recomputes, S * sizeof(long long));
-  zero(h->d_path_batches, 3 * S * sizeof(long long));
-  zero(h->d_init_moves, S * sizeof(long long));
-  zero(h->d_drift, S * sizeof(double));
-  zero(h->d_ctrl, 4 * sizeof(int32_t));
-  zero(h->d_ex_index, sizeof(long long));
-  if (ce == cudaSuccess) ce = cudaMemset(h->d_rt_last, 0xff, S * sizeof(int32_t));   // -1: no extreme seen yet
-  zero(h->d_rt_count, S * sizeof(long long));
-  zero(h->d_ex_att, std::max(h->h - 1, 1) * sizeof(unsigned long long));
-  zero(h->d_ex_acc, std::max(h->h - 1, 1) * sizeof(unsigned long long));
+  up(h->arena + h->small_begin, block.data(), block.size());
+  if (ce == cudaSuccess) ce = cudaMemsetAsync(h->d_rt_last, 0xff, S * sizeof(int32_t), h->stream);   // -1: none seen yet
   up(h->d_starts, h->starts.data(), h->h * sizeof(int32_t));
   if (h->part) {
     up(h->d_gid, h->gid_host.data(), S * sizeof(int32_t));
     up(h->d_pos_of, h->pos_host.data(), h->S_global * sizeof(int32_t));
   }
   if (g.kind == 1) {
-    std::vector<float> jf(h->tab_J.size());
     for (size_t t = 0; t < jf.size(); ++t) jf[t] = (float)h->tab_J[t];
     up(h->d_tab_nbr, h->tab_nbr.data(), h->tab_nbr.size() * sizeof(int32_t));
     up(h->d_tab_Jf, jf.data(), jf.size() * sizeof(float));
     up(h->d_tab_Jd, h->tab_J.data(), h->tab_J.size() * sizeof(double));
   }
-  if (ce == cudaSuccess) ce = cudaDeviceSynchronize();
+  if (ce == cudaSuccess) ce = cudaStreamSynchronize(h->stream);
   if (ce != cudaSuccess) {
     g_last_error = std::string("initial upload: ") + cudaGetErrorString(ce);
     rewl_destroy(h);
@@ -922,20 +1002,16 @@ static rewl_status enqueue_intervals(rewl_handle* h, int n) {
   return REWL_OK;
 }
 
-static rewl_status fill_stats(rewl_handle* h, rewl_stage_stats* out, int intervals, long long moves,
-                              int halved, double ms) {
+static void fill_stats(rewl_handle* h, const Walkers& w, rewl_stage_stats* out, int intervals, long long moves,
+                       int halved, double ms) {
   const size_t S = h->S;
-  std::vector<long long> acc(S);
-  std::vector<double> lnf(S), drift(S);
-  std::vector<unsigned long long> att(std::max(h->h - 1, 1)), ex(std::max(h->h - 1, 1));
-  CUDA_TRY(h, cudaMemcpyAsync(acc.data(), h->d_accepts, S * sizeof(long long), cudaMemcpyDeviceToHost, h->stream));
-  CUDA_TRY(h, cudaMemcpyAsync(lnf.data(), h->d_lnf, S * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
-  CUDA_TRY(h, cudaMemcpyAsync(drift.data(), h->d_drift, S * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
-  CUDA_TRY(h, cudaMemcpyAsync(att.data(), h->d_ex_att, att.size() * sizeof(unsigned long long), cudaMemcpyDeviceToHost, h->stream));
-  CUDA_TRY(h, cudaMemcpyAsync(ex.data(), h->d_ex_acc, ex.size() * sizeof(unsigned long long), cudaMemcpyDeviceToHost, h->stream));
-  CUDA_TRY(h, cudaStreamSynchronize(h->stream));
+  const long long* acc = w.at(h->d_accepts);
+  const double* lnf = w.at(h->d_lnf);
+  const double* drift = w.at(h->d_drift);
+  const unsigned long long* att = w.at(h->d_ex_att);
+  const unsigned long long* ex = w.at(h->d_ex_acc);
   long long tot_acc = 0;
-  for (auto v : acc) tot_acc += v;
+  for (size_t s = 0; s < S; ++s) tot_acc += acc[s];
   unsigned long long ta = 0, tx = 0;
   if (h->h > 1)
     for (int k = 0; k < h->h - 1; ++k) {
@@ -968,16 +1044,12 @@ static rewl_status fill_stats(rewl_handle* h, rewl_stage_stats* out, int interva
   h->prev_accepts = tot_acc;
   h->prev_ex_att = ta;
   h->prev_ex_acc = tx;
-  return REWL_OK;
 }
 
-static rewl_status read_stage(rewl_handle* h, std::vector<int32_t>& stage, std::vector<double>& lnf) {
-  stage.resize(h->S);
-  lnf.resize(h->S);
-  CUDA_TRY(h, cudaMemcpyAsync(stage.data(), h->d_stage, h->S * sizeof(int32_t), cudaMemcpyDeviceToHost, h->stream));
-  CUDA_TRY(h, cudaMemcpyAsync(lnf.data(), h->d_lnf, h->S * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
-  CUDA_TRY(h, cudaStreamSynchronize(h->stream));
-  return REWL_OK;
+static int count_halved(rewl_handle* h, const Walkers& before, const Walkers& after) {
+  int n = 0;
+  for (int i = 0; i < h->S; ++i) n += after.at(h->d_stage)[i] - before.at(h->d_stage)[i];
+  return n;
 }
 
 rewl_status rewl_run_intervals(rewl_handle* h, int n, rewl_stage_stats* stats) {
@@ -990,21 +1062,18 @@ rewl_status rewl_run_intervals(rewl_handle* h, int n, rewl_stage_stats* stats) {
     if (s != REWL_OK) return s;
   }
   const auto t0 = std::chrono::steady_clock::now();
-  std::vector<int32_t> st0, st1;
-  std::vector<double> l0, l1;
+  Walkers before, after;
   if (stats) {
-    s = read_stage(h, st0, l0);
+    s = before.read(h, false);
     if (s != REWL_OK) return s;
   }
   s = enqueue_intervals(h, n);
   if (s != REWL_OK) return s;
   if (stats) {
-    s = read_stage(h, st1, l1);
+    s = after.read(h, false);
     if (s != REWL_OK) return s;
-    int halved = 0;
-    for (int i = 0; i < h->S; ++i) halved += st1[i] - st0[i];
     const double ms = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
-    return fill_stats(h, stats, n, (long long)n * h->exchange_interval * h->S, halved, ms);
+    fill_stats(h, after, stats, n, (long long)n * h->exchange_interval * h->S, count_halved(h, before, after), ms);
   }
   return REWL_OK;
 }
@@ -1018,9 +1087,8 @@ rewl_status rewl_run_stage(rewl_handle* h, rewl_stage_stats* stats) {
     if (s != REWL_OK) return s;
   }
   const auto t0 = std::chrono::steady_clock::now();
-  std::vector<int32_t> st0, st;
-  std::vector<double> l0, l;
-  s = read_stage(h, st0, l0);
+  Walkers before, now;
+  s = before.read(h, false);
   if (s != REWL_OK) return s;
   long long moves_per_walker = 0;
   int intervals = 0;
@@ -1032,11 +1100,11 @@ rewl_status rewl_run_stage(rewl_handle* h, rewl_stage_stats* stats) {
     if (s != REWL_OK) return s;
     intervals += chunk;
     moves_per_walker += (long long)chunk * h->exchange_interval;
-    s = read_stage(h, st, l);
+    s = now.read(h, false);
     if (s != REWL_OK) return s;
     bool all = true;
     for (int i = 0; i < h->S; ++i)
-      if (l0[i] >= h->lnf_final && st[i] <= st0[i]) all = false;
+      if (before.at(h->d_lnf)[i] >= h->lnf_final && now.at(h->d_stage)[i] <= before.at(h->d_stage)[i]) all = false;
     if (all) break;
     const double secs = std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();
     if ((h->max_moves_per_stage > 0 && moves_per_walker >= h->max_moves_per_stage) ||
@@ -1046,11 +1114,8 @@ rewl_status rewl_run_stage(rewl_handle* h, rewl_stage_stats* stats) {
     }
     chunk = std::min(chunk * 2, 64);
   }
-  int halved = 0;
-  for (int i = 0; i < h->S; ++i) halved += st[i] - st0[i];
   const double ms = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
-  s = fill_stats(h, stats, intervals, moves_per_walker * h->S, halved, ms);
-  if (s != REWL_OK) return s;
+  fill_stats(h, now, stats, intervals, moves_per_walker * h->S, count_halved(h, before, now), ms);
   if (capped) return fail(h, REWL_ETIMEOUT, "stage ended by max_moves_per_stage or timeout_s");
   return REWL_OK;
 }
@@ -1070,7 +1135,12 @@ rewl_status rewl_exchange(rewl_handle* h, rewl_stage_stats* stats) {
   ea.key1 = h->key1;
   ea.traj = h->traj ? 1 : 0;
   CUDA_TRY(h, launch_exchange(ea, h->stream));
-  if (stats) return fill_stats(h, stats, 0, 0, 0, 0.0);
+  if (stats) {
+    Walkers w;
+    s = w.read(h, false);
+    if (s != REWL_OK) return s;
+    fill_stats(h, w, stats, 0, 0, 0, 0.0);
+  }
   return REWL_OK;
 }
 
@@ -1131,22 +1201,19 @@ rewl_status rewl_stitch_device(const double* frag, const int32_t* starts_host, i
   a.W = W;
   a.B = B;
   a.out = out;
-  int32_t* d_starts = nullptr;
-  double* d_avg = nullptr;
-  int32_t* d_bstar = nullptr;
-  cudaError_t e = cudaMallocAsync(&d_starts, sizeof(int32_t) * n_windows, st);
-  if (e == cudaSuccess) e = cudaMallocAsync(&d_avg, sizeof(double) * (size_t)n_windows * W, st);
-  if (e == cudaSuccess && !bstar_out) e = cudaMallocAsync(&d_bstar, sizeof(int32_t) * std::max(n_windows - 1, 1), st);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(d_starts, starts_host, sizeof(int32_t) * n_windows, cudaMemcpyHostToDevice, st);
+  auto align = [](size_t n) { return (n + 255) & ~(size_t)255; };
+  const size_t avg_bytes = align(sizeof(double) * (size_t)n_windows * W), list = align(sizeof(int32_t) * (size_t)n_windows);
+  void* scratch = nullptr;
+  cudaError_t e = pool_alloc(&scratch, avg_bytes + 2 * list, st);
   if (e == cudaSuccess) {
+    a.avg = static_cast<double*>(scratch);
+    int32_t* d_starts = reinterpret_cast<int32_t*>(static_cast<unsigned char*>(scratch) + avg_bytes);
     a.starts = d_starts;
-    a.avg = d_avg;
-    a.bstar = bstar_out ? bstar_out : d_bstar;
-    e = launch_merge(a, st);
+    a.bstar = bstar_out ? bstar_out : d_starts + list / sizeof(int32_t);
+    e = cudaMemcpyAsync(d_starts, starts_host, sizeof(int32_t) * n_windows, cudaMemcpyHostToDevice, st);
+    if (e == cudaSuccess) e = launch_merge(a, st);
   }
-  if (d_starts) cudaFreeAsync(d_starts, st);
-  if (d_avg) cudaFreeAsync(d_avg, st);
-  if (d_bstar) cudaFreeAsync(d_bstar, st);
+  pool_free(scratch, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) return fail(nullptr, REWL_ECUDA, std::string("stitch: ") + cudaGetErrorString(e));
   return REWL_OK;
@@ -1160,19 +1227,21 @@ rewl_status rewl_thermo(const double* lng, const double* centres, int B, double 
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
   double* d = nullptr;
   const size_t bytes = sizeof(double) * (2 * (size_t)B + 4 * (size_t)nT);
-  cudaError_t e = cudaMallocAsync(&d, bytes, st);
+  cudaError_t e = pool_alloc(reinterpret_cast<void**>(&d), bytes, st);
   if (e != cudaSuccess) return fail(nullptr, REWL_ENOMEM, "thermo scratch allocation failed");
+  std::vector<double> out(3 * (size_t)nT);
   double *dl = d, *dE = d + B, *dT = d + 2 * B, *dU = dT + nT, *dC = dU + nT, *dZ = dC + nT;
   e = cudaMemcpyAsync(dl, lng, sizeof(double) * B, cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess) e = cudaMemcpyAsync(dE, centres, sizeof(double) * B, cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess) e = cudaMemcpyAsync(dT, T, sizeof(double) * nT, cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess) e = launch_thermo(dl, dE, B, n_spins, dT, nT, dU, dC, dZ, st);
-  if (e == cudaSuccess && U) e = cudaMemcpyAsync(U, dU, sizeof(double) * nT, cudaMemcpyDeviceToHost, st);
-  if (e == cudaSuccess && C) e = cudaMemcpyAsync(C, dC, sizeof(double) * nT, cudaMemcpyDeviceToHost, st);
-  if (e == cudaSuccess && lnZ) e = cudaMemcpyAsync(lnZ, dZ, sizeof(double) * nT, cudaMemcpyDeviceToHost, st);
-  cudaFreeAsync(d, st);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(out.data(), dU, sizeof(double) * out.size(), cudaMemcpyDeviceToHost, st);
+  pool_free(d, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) return fail(nullptr, REWL_ECUDA, std::string("thermo: ") + cudaGetErrorString(e));
+  if (U) std::copy_n(out.begin(), nT, U);
+  if (C) std::copy_n(out.begin() + nT, nT, C);
+  if (lnZ) std::copy_n(out.begin() + 2 * (size_t)nT, nT, lnZ);
   return REWL_OK;
 }
 
@@ -1180,13 +1249,13 @@ rewl_status rewl_peak_temperature(const double* T, const double* C, int nT, doub
   if (!T || !C || !T_peak || nT < 1) return fail(nullptr, REWL_EINVAL, "bad peak arguments");
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
   double* d = nullptr;
-  cudaError_t e = cudaMallocAsync(&d, sizeof(double) * (2 * (size_t)nT + 1), st);
+  cudaError_t e = pool_alloc(reinterpret_cast<void**>(&d), sizeof(double) * (2 * (size_t)nT + 1), st);
   if (e != cudaSuccess) return fail(nullptr, REWL_ENOMEM, "peak scratch allocation failed");
   e = cudaMemcpyAsync(d, T, sizeof(double) * nT, cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess) e = cudaMemcpyAsync(d + nT, C, sizeof(double) * nT, cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess) e = launch_peak(d, d + nT, nT, d + 2 * nT, st);
   if (e == cudaSuccess) e = cudaMemcpyAsync(T_peak, d + 2 * nT, sizeof(double), cudaMemcpyDeviceToHost, st);
-  cudaFreeAsync(d, st);
+  pool_free(d, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) return fail(nullptr, REWL_ECUDA, std::string("peak: ") + cudaGetErrorString(e));
   return REWL_OK;
@@ -1257,44 +1326,34 @@ rewl_status rewl_get_walkers(rewl_handle* h, double* lng, uint32_t* H, double* E
   rewl_status s = check_ready(h);
   if (s != REWL_OK) return s;
   const size_t S = h->S, W = h->W;
-  cudaStream_t st = h->stream;
-  if (lng) {
-    if (h->traj) {
-      CUDA_TRY(h, cudaMemcpyAsync(lng, h->d_lng, S * W * sizeof(double), cudaMemcpyDeviceToHost, st));
-    } else {
-      std::vector<long long> t(S * W);
-      CUDA_TRY(h, cudaMemcpyAsync(t.data(), h->d_lng_fx, S * W * sizeof(long long), cudaMemcpyDeviceToHost, st));
-      CUDA_TRY(h, cudaStreamSynchronize(st));
-      for (size_t i = 0; i < S * W; ++i) lng[i] = (double)t[i] * kLngUnit;
+  Walkers w;
+  s = w.read(h, lng || H);
+  if (s != REWL_OK) return s;
+  auto give = [&](auto* out, const auto* d, size_t count) {
+    if (out) std::memcpy(out, w.at(d), count * sizeof *out);
+  };
+  if (lng && h->traj) give(lng, h->d_lng, S * W);
+  if (lng && !h->traj) {
+    const long long* t = w.at(h->d_lng_fx);
+    for (size_t i = 0; i < S * W; ++i) lng[i] = (double)t[i] * kLngUnit;
+  }
+  give(H, h->d_H, S * W);
+  if (h->traj) {
+    give(E, h->d_E, S);
+    give(bin, h->d_bin, S);
+  } else {
+    const long long* f = w.at(h->d_efx);
+    for (size_t i = 0; i < S; ++i) {
+      if (E) E[i] = h->e_min + h->dE * ((double)f[i] / kEnergyScale);
+      if (bin) bin[i] = (int32_t)(f[i] >> 32);
     }
   }
-  if (H) CUDA_TRY(h, cudaMemcpyAsync(H, h->d_H, S * W * sizeof(uint32_t), cudaMemcpyDeviceToHost, st));
-  if (E || bin) {
-    std::vector<double> e(S);
-    std::vector<int32_t> b(S);
-    if (h->traj) {
-      CUDA_TRY(h, cudaMemcpyAsync(e.data(), h->d_E, S * sizeof(double), cudaMemcpyDeviceToHost, st));
-      CUDA_TRY(h, cudaMemcpyAsync(b.data(), h->d_bin, S * sizeof(int32_t), cudaMemcpyDeviceToHost, st));
-      CUDA_TRY(h, cudaStreamSynchronize(st));
-    } else {
-      std::vector<long long> f(S);
-      CUDA_TRY(h, cudaMemcpyAsync(f.data(), h->d_efx, S * sizeof(long long), cudaMemcpyDeviceToHost, st));
-      CUDA_TRY(h, cudaStreamSynchronize(st));
-      for (size_t i = 0; i < S; ++i) {
-        e[i] = h->e_min + h->dE * ((double)f[i] / kEnergyScale);
-        b[i] = (int32_t)(f[i] >> 32);
-      }
-    }
-    if (E) std::memcpy(E, e.data(), S * sizeof(double));
-    if (bin) std::memcpy(bin, b.data(), S * sizeof(int32_t));
-  }
-  if (lnf) CUDA_TRY(h, cudaMemcpyAsync(lnf, h->d_lnf, S * sizeof(double), cudaMemcpyDeviceToHost, st));
-  if (replica) CUDA_TRY(h, cudaMemcpyAsync(replica, h->d_perm, S * sizeof(int32_t), cudaMemcpyDeviceToHost, st));
-  if (stage) CUDA_TRY(h, cudaMemcpyAsync(stage, h->d_stage, S * sizeof(int32_t), cudaMemcpyDeviceToHost, st));
-  if (accepts) CUDA_TRY(h, cudaMemcpyAsync(accepts, h->d_accepts, S * sizeof(long long), cudaMemcpyDeviceToHost, st));
-  if (steps) CUDA_TRY(h, cudaMemcpyAsync(steps, h->d_steps, S * sizeof(long long), cudaMemcpyDeviceToHost, st));
-  if (init_moves) CUDA_TRY(h, cudaMemcpyAsync(init_moves, h->d_init_moves, S * sizeof(long long), cudaMemcpyDeviceToHost, st));
-  CUDA_TRY(h, cudaStreamSynchronize(st));
+  give(lnf, h->d_lnf, S);
+  give(replica, h->d_perm, S);
+  give(stage, h->d_stage, S);
+  give(accepts, h->d_accepts, S);
+  give(steps, h->d_steps, S);
+  give(init_moves, h->d_init_moves, S);
   return REWL_OK;
 }
 
@@ -1310,10 +1369,10 @@ rewl_status rewl_get_spins(rewl_handle* h, double* spins) {
     // device codes -> the FP32 spins the walkers see (decoded on the device) -> host FP64 planes
     float* d = nullptr;
     std::vector<float> t(n);
-    CUDA_TRY(h, cudaMallocAsync(&d, n * sizeof(float), h->stream));
+    CUDA_TRY(h, pool_alloc(reinterpret_cast<void**>(&d), n * sizeof(float), h->stream));
     CUDA_TRY(h, launch_decode_spins(static_cast<const float2*>(h->d_spins), (size_t)h->S, h->N, d, h->stream));
     CUDA_TRY(h, cudaMemcpyAsync(t.data(), d, n * sizeof(float), cudaMemcpyDeviceToHost, h->stream));
-    CUDA_TRY(h, cudaFreeAsync(d, h->stream));
+    pool_free(d, h->stream);
     CUDA_TRY(h, cudaStreamSynchronize(h->stream));
     for (size_t i = 0; i < n; ++i) spins[i] = t[i];
   }
@@ -1371,13 +1430,13 @@ rewl_status rewl_get_neighbours(rewl_handle* h, int32_t* nbr, double* J) {
   const size_t n = (size_t)h->z * h->N;
   int32_t* dn = nullptr;
   double* dj = nullptr;
-  CUDA_TRY(h, cudaMallocAsync(&dn, n * sizeof(int32_t), h->stream));
-  CUDA_TRY(h, cudaMallocAsync(&dj, n * sizeof(double), h->stream));
+  CUDA_TRY(h, pool_alloc(reinterpret_cast<void**>(&dn), n * sizeof(int32_t), h->stream));
+  CUDA_TRY(h, pool_alloc(reinterpret_cast<void**>(&dj), n * sizeof(double), h->stream));
   CUDA_TRY(h, launch_neighbour_dump(h->geo, dn, dj, h->stream));
   CUDA_TRY(h, cudaMemcpyAsync(nbr, dn, n * sizeof(int32_t), cudaMemcpyDeviceToHost, h->stream));
   CUDA_TRY(h, cudaMemcpyAsync(J, dj, n * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
-  CUDA_TRY(h, cudaFreeAsync(dn, h->stream));
-  CUDA_TRY(h, cudaFreeAsync(dj, h->stream));
+  pool_free(dn, h->stream);
+  pool_free(dj, h->stream);
   CUDA_TRY(h, cudaStreamSynchronize(h->stream));
   return REWL_OK;
 }
@@ -1387,11 +1446,11 @@ rewl_status rewl_replica_energies(rewl_handle* h, double* E) {
   if (s != REWL_OK) return s;
   if (!E) return fail(h, REWL_EINVAL, "E is NULL");
   double* d = nullptr;
-  CUDA_TRY(h, cudaMallocAsync(&d, h->S * sizeof(double), h->stream));
+  CUDA_TRY(h, pool_alloc(reinterpret_cast<void**>(&d), h->S * sizeof(double), h->stream));
   const WalkerArgs a = walker_args(h, false, false, 0);
   CUDA_TRY(h, launch_energies(a, h->S, h->traj, d, h->stream));
   CUDA_TRY(h, cudaMemcpyAsync(E, d, h->S * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
-  CUDA_TRY(h, cudaFreeAsync(d, h->stream));
+  pool_free(d, h->stream);
   CUDA_TRY(h, cudaStreamSynchronize(h->stream));
   return REWL_OK;
 }

@@ -18,6 +18,13 @@ struct NvtxRange {
   NvtxRange& operator=(const NvtxRange&) = delete;
 };
 
+// The library's stream-ordered memory pool of the current device (api.cu).  pool_free orders the free after the
+// stream's work; every handle and model retains the pool while it lives.
+cudaError_t pool_alloc(void** p, size_t bytes, cudaStream_t stream);
+void pool_free(void* p, cudaStream_t stream);
+void pool_retain();
+void pool_release();
+
 struct JobView {
   int kind, N, z, L, S, W, h, m, n_shells;
   bool traj, pipe, initialized, broken, part;

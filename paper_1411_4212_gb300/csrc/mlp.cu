@@ -794,16 +794,18 @@ rewl_status malloc_dev(rewl_mlp* m, T** p, size_t count) {
   return REWL_OK;
 }
 
-// device scratch of one call, freed on return
+// device scratch of one call, freed on return in the order of the model's stream
 struct Scratch {
+  cudaStream_t stream;
   std::vector<void*> ptrs;
+  explicit Scratch(rewl_mlp* m) : stream(m->stream) {}
   ~Scratch() {
-    for (void* p : ptrs) cudaFree(p);
+    for (void* p : ptrs) pool_free(p, stream);
   }
   template <class T>
   cudaError_t get(T** p, size_t count) {
     void* q = nullptr;
-    const cudaError_t e = cudaMalloc(&q, std::max<size_t>(count, 1) * sizeof(T));
+    const cudaError_t e = pool_alloc(&q, std::max<size_t>(count, 1) * sizeof(T), stream);
     if (e == cudaSuccess) {
       ptrs.push_back(q);
       *p = static_cast<T*>(q);
@@ -866,6 +868,7 @@ rewl_status loss_and_grad(rewl_mlp* m, const float* dx, const float* dt, const i
 
 struct Corpus {
   Scratch sc;
+  explicit Corpus(rewl_mlp* m) : sc(m) {}
   float *x = nullptr, *t = nullptr, *y = nullptr, *dy = nullptr;
   int* seg = nullptr;
   double* loss = nullptr;
@@ -898,6 +901,7 @@ extern "C" rewl_status rewl_mlp_create(const float* in_shift, const float* in_sc
     if (!std::isfinite(in_shift[k]) || !std::isfinite(in_scale[k]) || in_scale[k] == 0.0f)
       return mfail(nullptr, REWL_EINVAL, "input normalisation must be finite with nonzero scales");
   auto* m = new rewl_mlp();
+  pool_retain();
   for (int k = 0; k < kIn; ++k) {
     m->net.shift[k] = in_shift[k];
     m->net.scale[k] = in_scale[k];
@@ -913,6 +917,7 @@ extern "C" rewl_status rewl_mlp_create(const float* in_shift, const float* in_sc
   if (ce == cudaSuccess)
     ce = cudaFuncSetAttribute(mlp_dw_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(DwSmem));
   if (ce != cudaSuccess) {
+    pool_release();
     delete m;
     return mfail(nullptr, REWL_ECUDA, std::string("CUDA set-up: ") + cudaGetErrorString(ce));
   }
@@ -977,7 +982,7 @@ extern "C" rewl_status rewl_mlp_forward(rewl_mlp* m, const float* x, int64_t n, 
   rewl_status s = check_mlp(m);
   if (s != REWL_OK) return s;
   if (!x || !y || n < 1) return mfail(m, REWL_EINVAL, "bad forward arguments");
-  Corpus c;
+  Corpus c(m);
   MCUDA(m, c.sc.get(&c.x, (size_t)n * kIn));
   MCUDA(m, c.sc.get(&c.y, (size_t)n));
   MCUDA(m, cudaMemcpyAsync(c.x, x, sizeof(float) * (size_t)n * kIn, cudaMemcpyHostToDevice, m->stream));
@@ -995,7 +1000,7 @@ extern "C" rewl_status rewl_mlp_gradient(rewl_mlp* m, const float* x, const floa
   if (!x || !target) return mfail(m, REWL_EINVAL, "NULL corpus");
   s = check_segments(run_offsets, n_runs, run_offsets ? run_offsets[n_runs] : 0);
   if (s != REWL_OK) return s;
-  Corpus c;
+  Corpus c(m);
   s = upload_corpus(m, c, x, target, run_offsets, n_runs);
   if (s != REWL_OK) return s;
   double* d_loss = nullptr;
@@ -1016,7 +1021,7 @@ extern "C" rewl_status rewl_mlp_train(rewl_mlp* m, const float* x, const float* 
   s = check_segments(run_offsets, n_runs, run_offsets ? run_offsets[n_runs] : 0);
   if (s != REWL_OK) return s;
   const long long n = run_offsets[n_runs];
-  Corpus c;
+  Corpus c(m);
   s = upload_corpus(m, c, x, target, run_offsets, n_runs);
   if (s != REWL_OK) return s;
   double* d_loss = nullptr;      // loss before each step
@@ -1088,5 +1093,6 @@ extern "C" void rewl_mlp_destroy(rewl_mlp* m) {
   if (!m) return;
   if (!m->broken) cudaStreamSynchronize(m->stream);
   for (void* p : m->allocations) cudaFree(p);
+  pool_release();
   delete m;
 }
