@@ -55,6 +55,15 @@ __device__ __forceinline__ double exp_fp64(double x, const ExpCoeffs& c) {
   return __dmul_rn(p, two_k);
 }
 
+// FP64 numbers as signed integers in the same order (NaN at the ends by its sign), and back.
+__device__ __forceinline__ long long order_key(double v) {
+  const long long b = __double_as_longlong(v);
+  return b ^ ((b >> 63) & 0x7fffffffffffffffLL);
+}
+__device__ __forceinline__ double order_value(long long k) {
+  return __longlong_as_double(k ^ ((k >> 63) & 0x7fffffffffffffffLL));
+}
+
 // Half-unit coordinates (X, Y, Z) of bcc site i = 2 (x + L (y + L z)) + s: (2x+s, 2y+s, 2z+s).
 // Division by L via the multiplier ceil(2^32 / L), exact for cell indices below 2^32 / L.
 __device__ __forceinline__ void bcc_coords(int i, int L, uint32_t divL, int& X, int& Y, int& Z) {

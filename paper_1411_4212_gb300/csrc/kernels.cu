@@ -530,15 +530,6 @@ __device__ double block_sum(double v, double* red) {
   return r;
 }
 
-// FP64 numbers as signed integers in the same order (NaN at the ends by its sign), and back.
-__device__ __forceinline__ long long order_key(double v) {
-  const long long b = __double_as_longlong(v);
-  return b ^ ((b >> 63) & 0x7fffffffffffffffLL);
-}
-__device__ __forceinline__ double order_value(long long k) {
-  return __longlong_as_double(k ^ ((k >> 63) & 0x7fffffffffffffffLL));
-}
-
 // e^x for x <= 0 (0 below -708, NaN for NaN) in integer arithmetic, within about a unit in the last place:
 // this GPU issues less than two FP64 operations per clock and SM, but 64-bit products of integers at a tenth
 // of its FP32 rate.  -x log2(e) = n + j/64 + r in 2^-53 units, r < 1/64;  e^x = 2^-n 2^(-j/64) 2^-r with the

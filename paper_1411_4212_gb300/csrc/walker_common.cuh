@@ -73,6 +73,7 @@ struct SpinPlanes {
     y[i] = vy;
     z[i] = vz;
   }
+  __device__ __forceinline__ Real component(int i, int c) const { return x[i + c * (y - x)]; }
 };
 
 struct SpinCodes {

@@ -9,15 +9,13 @@
 //     resolved while batch b+1 reads the lattice) and the earlier moves of batch b+1 that sit on the
 //     same site or a neighbouring one;
 //   resolver: a move whose mask meets a move accepted since the lattice was read is corrected
-//     exactly (production: from the move batches; trajectory: re-evaluated on the current lattice);
+//     exactly (production: from the move batches; trajectory: summed again on the current lattice);
 //     then accept with min[1, g(E)/g(E')] (reject outside the window) and add ln f to ln g and 1 to
 //     H at the resulting state.
 // The owner table may alias sites (hashed): an alias names a move that cannot change the field; the
-// production producer sorts such bits out by the distance of the sites.  Two record buffers alternate; named barriers READY(b mod 2) and DONE(b mod 2)
-// order the hand-over, so the producer reads the lattice only after every move of batch b-1 has been
-// written.
-#include <cstring>
-
+// producer sorts such bits out by the distance of the sites.  Two record buffers alternate; named barriers
+// READY(b mod 2) and DONE(b mod 2) order the hand-over, so the producer reads the lattice only after every
+// move of batch b-1 has been written.
 #include "walker_common.cuh"
 
 namespace rewl {
@@ -53,22 +51,23 @@ struct alignas(16) MoveBatch {
                          // increment is a bin or more (count)
 };
 
-// Trajectory: one move.
-struct alignas(16) TrajRec {
-  double dE;
-  double u;
-  uint32_t cprev, ccur;
-  int site, pad;
-  double nx, ny, nz, pad2;
+// Trajectory: one batch of 32 trial moves, an array per quantity.
+struct alignas(16) TrajBatch {
+  double dE[32], u[32];
+  double nx[32], ny[32], nz[32];
+  int4 move[32];         // site | half-unit coordinates X | Y << 10 | Z << 20 | ln u to 4e-6 (1 where u is too small
+                         // for it) | dE in 2^-24 bins
+  int4 marks[32];        // moves of batch b-1, earlier moves of this batch that touch this one; the same as the
+                         // owner table has them (with the aliases), for the count of recomputed moves
 };
 
 // Bytes of the two move batches in flight.
 __host__ __device__ constexpr size_t batch_bytes(bool traj) {
-  return traj ? 64 * sizeof(TrajRec) : 2 * sizeof(MoveBatch);
+  return traj ? 2 * sizeof(TrajBatch) : 2 * sizeof(MoveBatch);
 }
 
 // Local field of (X, Y, Z) by one lane over all slots in canonical order, with the owner-table
-// words of the site's neighbours OR-ed into own[shell].
+// words of the site's neighbours OR-ed into touch[shell] (trajectory: touch[0]).
 template <bool kTraj, int NSH, class Lat>
 __device__ __forceinline__ void field_one_lane(const Lat& lat, int X, int Y, int Z, int L, const typename Mode<kTraj>::Real (&Jsh)[4],
                                                typename Mode<kTraj>::Real& hx, typename Mode<kTraj>::Real& hy,
@@ -117,8 +116,8 @@ __device__ __forceinline__ void field_one_lane(const Lat& lat, int X, int Y, int
       tz[T.sh[j]] += vz;
     }
     const uint2 o = own[n & omask];
-    touch[T.sh[j]].x |= o.x;
-    touch[T.sh[j]].y |= o.y;
+    touch[kTraj ? 0 : T.sh[j]].x |= o.x;
+    touch[kTraj ? 0 : T.sh[j]].y |= o.y;
   }
   if constexpr (!kTraj) {
 #pragma unroll
@@ -140,6 +139,53 @@ __device__ __forceinline__ int dq24_of(float dE, const Windows& w) {
   return __float2int_rn(p) + __float2int_rn(e);
 }
 
+// Trajectory mode.  dE in 2^-24 bins, at most kFarUnits = 64 bins either way (NaN: kFarUnits).
+constexpr int kFarUnits = 1 << 30;
+__device__ __forceinline__ int traj_units(double dE, double bin_units) {
+  const int q = __double2int_rn(dE * bin_units);
+  return dE == dE ? max(-kFarUnits, min(kFarUnits, q)) : kFarUnits;
+}
+// dE = -(S' - S) . h, one rounding per operation.
+__device__ __forceinline__ double traj_energy(double nx, double ny, double nz, double ox, double oy, double oz, double hx,
+                                              double hy, double hz) {
+  const double dx = __dsub_rn(nx, ox), dy = __dsub_rn(ny, oy), dz = __dsub_rn(nz, oz);
+  return -__dadd_rn(__dadd_rn(__dmul_rn(dx, hx), __dmul_rn(dy, hy)), __dmul_rn(dz, hz));
+}
+// dE of a move on the lattice as it is by a whole warp, in the producer's order: a product per lane, then the
+// component of the field per lane (the sums are as long as by one lane, the FP64 issue a fifth).
+template <int NSH>
+__device__ __forceinline__ double traj_again(const SpinPlanes<double>& lat, const uint32_t* off_s, const double* J_s,
+                                             int site, uint32_t coords, double nx, double ny, double nz, int L, int lane) {
+  constexpr int z = make_shells(NSH).z, kParts = (3 * z + 31) / 32;
+  double prod[kParts];
+#pragma unroll
+  for (int q = 0; q < kParts; ++q) {
+    const int i = min(q * 32 + lane, 3 * z - 1), j = i / 3;
+    int dx, dy, dz;
+    unpack_offset(off_s[j], dx, dy, dz);
+    const int n = bcc_offset_site((int)(coords & 1023u), (int)((coords >> 10) & 1023u), (int)(coords >> 20), dx, dy, dz, L);
+    prod[q] = __dmul_rn(J_s[j], lat.component(n, i - 3 * j));
+  }
+  const int c = lane % 3;
+  const double d = __dsub_rn(c == 0 ? nx : c == 1 ? ny : nz, lat.component(site, c));
+  double h = 0.0;
+#pragma unroll
+  for (int j = 0; j < z; ++j) {
+    // product 3 j + c: part (3 j + c) / 32 of lane (3 j + c) % 32
+    const int q0 = 3 * j / 32, q1 = (3 * j + 2) / 32;
+    double v = __shfl_sync(kFullMask, prod[q0], (3 * j + c) & 31);
+    if (q1 != q0) {
+      const double v1 = __shfl_sync(kFullMask, prod[q1], (3 * j + c) & 31);
+      v = 3 * j + c >= 32 * q1 ? v1 : v;
+    }
+    h = __dadd_rn(h, v);
+  }
+  const double p = __dmul_rn(d, h);
+  return -__dadd_rn(__dadd_rn(__shfl_sync(kFullMask, p, 0), __shfl_sync(kFullMask, p, 1)), __shfl_sync(kFullMask, p, 2));
+}
+// Order key of an entry of the ln g table; NaN above every number.
+__device__ __forceinline__ long long traj_key(double v) { return order_key(v == v ? v : fabs(v)); }
+
 // One exchange interval of walker slot `slot` by a group of nt threads (tid = 0..nt-1, nt a multiple
 // of 32, at least 64): warp 0 resolves, warp 1 produces, every warp loads and stores.  smem_raw is
 // the group's shared-memory arena (walker_pipe_smem_bytes), red holds nt/32 doubles.  Barrier
@@ -151,7 +197,7 @@ __device__ __forceinline__ void pipe_walk_slot(const WalkerArgs& a, const int sl
                                                const int tid, const int nt, const int bar_sync,
                                                const int bar_pair) {
   using Real = typename Mode<kTraj>::Real;
-  using Lng = typename Mode<kTraj>::Lng;
+  using Lng = long long;   // production: 2^-40 units; trajectory: the order key of the FP64 value
   const int kBarReady = bar_pair, kBarDone = bar_pair + 2;
   const int warp = tid >> 5, lane = tid & 31;
   const int N = a.geo.N, W = a.win.W, L = a.geo.L;
@@ -170,7 +216,7 @@ __device__ __forceinline__ void pipe_walk_slot(const WalkerArgs& a, const int sl
   p += 4 * kMaxSlotsPerSite;
   Real* J_s = reinterpret_cast<Real*>(p);
   p += sizeof(Real) * kMaxSlotsPerSite;
-  TrajRec* rec = reinterpret_cast<TrajRec*>(p);            // trajectory: [2][32]
+  TrajBatch* rec = reinterpret_cast<TrajBatch*>(p);        // trajectory: [2]
   MoveBatch* mb = reinterpret_cast<MoveBatch*>(p);         // production: [2]
   p += batch_bytes(kTraj);
   uint2* own = reinterpret_cast<uint2*>(p);
@@ -187,9 +233,9 @@ __device__ __forceinline__ void pipe_walk_slot(const WalkerArgs& a, const int sl
   const size_t lbase = (size_t)slot * W;
   for (int w = tid; w < W; w += nt) {
     if constexpr (kTraj)
-      lng_s[w] = (Lng)a.st.lng[lbase + w];
+      lng_s[w] = traj_key(a.st.lng[lbase + w]);
     else
-      lng_s[w] = (Lng)a.st.lng_fx[lbase + w];
+      lng_s[w] = a.st.lng_fx[lbase + w];
     H_s[w] = a.st.H[lbase + w];
   }
   for (int j = tid; j < kMaxSlotsPerSite; j += nt) {
@@ -203,6 +249,8 @@ __device__ __forceinline__ void pipe_walk_slot(const WalkerArgs& a, const int sl
   const int nb = (int)((moves + 31) / 32);
   const long long t0 = a.st.steps[slot];
   const uint2 key = make_uint2((uint32_t)global_slot(a.st, slot), a.key1);
+
+  const double bin_units = kTraj ? 16777216.0 / a.win.dE : 0.0;   // 2^-24 bins per unit of energy
 
   if (warp == 1) {
     // ------------------------------- producer -------------------------------
@@ -272,16 +320,33 @@ __device__ __forceinline__ void pipe_walk_slot(const WalkerArgs& a, const int sl
         cprev |= tprev[s2];
       }
       if constexpr (kTraj) {
-        TrajRec& r = rec[cur * 32 + lane];
-        const double dx = __dsub_rn(nx, ox), dy = __dsub_rn(ny, oy), dz = __dsub_rn(nz, oz);
-        r.dE = -__dadd_rn(__dadd_rn(__dmul_rn(dx, hx), __dmul_rn(dy, hy)), __dmul_rn(dz, hz));
-        r.u = u;
-        r.cprev = cprev;
-        r.ccur = ccur;
-        r.site = site;
-        r.nx = nx;
-        r.ny = ny;
-        r.nz = nz;
+        TrajBatch& m = rec[cur];
+        const double dE = traj_energy(nx, ny, nz, ox, oy, oz, hx, hy, hz);
+        const float lu = u > 0x1.0p-100 ? logf(__double2float_rn(u)) : 1.0f;
+        m.dE[lane] = dE;
+        m.u[lane] = u;
+        m.nx[lane] = nx;
+        m.ny[lane] = ny;
+        m.nz[lane] = nz;
+        m.move[lane] = make_int4(site, X | (Y << 10) | (Z << 20), __float_as_int(lu), traj_units(dE, bin_units));
+        __syncwarp();
+        // the table's bits without the aliases: moves on this site or on a neighbour
+        auto touching = [&](const TrajBatch& other, uint32_t bits) -> uint32_t {
+          uint32_t real = 0u;
+          for (; bits; bits &= bits - 1u) {
+            const int j = __ffs(bits) - 1;
+            const uint32_t q = (uint32_t)other.move[j].y;
+            int ex = abs((int)(q & 1023u) - X), ey = abs((int)((q >> 10) & 1023u) - Y), ez = abs((int)(q >> 20) - Z);
+            ex = min(ex, 2 * L - ex);
+            ey = min(ey, 2 * L - ey);
+            ez = min(ez, 2 * L - ez);
+            const int r2 = ex * ex + ey * ey + ez * ez;
+            real |= r2 == 0 || r2 == 3 || (NSH > 1 && r2 == 4) || (NSH > 2 && r2 == 8) || (NSH > 3 && r2 == 11) ? 1u << j : 0u;
+          }
+          return real;
+        };
+        m.marks[lane] = make_int4((int)(aliased ? touching(rec[cur ^ 1], cprev) : cprev),
+                                  (int)(aliased ? touching(m, ccur) : ccur), (int)cprev, (int)ccur);
       } else {
         MoveBatch& m = mb[cur];
         // (rounded subtractions: a plain one could fuse with the product that decoded the old spin)
@@ -346,87 +411,206 @@ __device__ __forceinline__ void pipe_walk_slot(const WalkerArgs& a, const int sl
   } else if (warp == 0) {
    if constexpr (kTraj) {
     // ------------------------ resolver (trajectory mode) ------------------------
+    // The walk in FP64 exactly as specified, one rounding per operation; but an FP64 operation takes 62 cycles,
+    // a division 550 and the specified exponential 34 operations in a row, so none of them sits on the chain
+    // from one accepted move to the next.  Lane k holds move k; a round finds the first move that is accepted,
+    // as in the production resolver below, from quantities that decide all but a few moves in 1e5:
+    //   - the walker's position to 2^-24 bins in integers (taken afresh from E every batch, off by at most one
+    //     unit, then half a unit per accepted move): its bin is certain unless it lies within kEdge units of a
+    //     bin's edge;
+    //   - ln g(now) - ln u to kTol (ln u is good to 4e-6, the sums below 1e9 to 1e-6): the move is accepted if
+    //     ln g(target) is below, rejected if above by more.
+    // A move that this leaves open, or whose dE is of an older lattice, is taken when its turn comes: its dE is
+    // summed again, and the specified operations decide.  E and the exact ln g are carried beside the chain.  A
+    // bin's ln g grows by a rounded addition of ln f per move; where no sum of this call can round (grid) that is
+    // one product and sum, else the additions are made when the walker leaves the bin.  The table holds order
+    // keys, so comparisons are integer ones.
+    // Measured, bcc L = 16, 2 shells, 64 walkers: 18.3 ms per 10^4 moves with every move decided in turn, 2.8 ms
+    // so (slowest walker, 30 of 32 moves accepted: 17,500 cycles per batch, 370 per accepted move and 2,100 per dE
+    // summed again; the producer's 12,600, mostly FP64 issue at 17 cycles per warp instruction, come next).
+    constexpr int kBin = 1 << 24, kEdge = 64;
+    constexpr double kTol = 1e-5;
+    constexpr uint32_t kNoKey = 0xffffffffu, kRare = 0x07fffffeu, kPayload = 0x07ffffffu;
     double E = a.st.E[slot];
-    int bcur = a.st.bin[slot];
-    const double lnf = a.st.lnf[slot];
-    const bool frozen = !(lnf >= a.lnf_final);
-    const bool bad = (unsigned)(bcur - wlo) >= (unsigned)W;
-    if (bad && lane == 0) atomicExch(a.st.ctrl + 0, kErrOutOfWindow);
-    double lng_cur = bad ? 0.0 : lng_s[bcur - wlo];
-    uint32_t h_cur = bad ? 0u : H_s[bcur - wlo];
-    constexpr int kWords = (int)(sizeof(TrajRec) / sizeof(int4));
+    int r = a.st.bin[slot] - wlo;
+    const double lnf0 = a.st.lnf[slot];
+    const bool frozen = !(lnf0 >= a.lnf_final);
+    const double lnf = frozen ? 0.0 : lnf0;
+    const bool bad = (unsigned)r >= (unsigned)W;
+    if (bad) {
+      if (lane == 0) atomicExch(a.st.ctrl + 0, kErrOutOfWindow);
+      r = 0;                                  // no move is made
+    }
+    const double lane_lnf = (double)lane * lnf;
+    const uint32_t lane_key = (uint32_t)lane << 27;
+    // grid: every sum that ln g can reach in this call is exact, as all entries and ln f are multiples of 2^low
+    // and nothing gets as large as 2^(low + 53)
+    bool grid;
+    {
+      // exponent and lowest set bit (both biased) of an entry; 0 takes no part, what is not a plain number none
+      int high = 0, low = 4096;
+      auto note = [&](double v) {
+        const unsigned long long m = (unsigned long long)__double_as_longlong(v) & 0x7fffffffffffffffULL;
+        const int ex = (int)(m >> 52);
+        const unsigned long long f = m & 0xfffffffffffffULL;
+        high = max(high, ex);
+        low = m == 0ULL ? low : ex == 0 || ex == 2047 ? -4096 : min(low, f ? ex - 53 + __ffsll((long long)f) : ex);
+      };
+      for (int w = lane; w < W; w += 32) note(order_value(lng_s[w]));
+      high = __reduce_max_sync(kFullMask, high);
+      low = __reduce_min_sync(kFullMask, low);
+      note(lnf);
+      // |ln g| < 2^(high - 1022) + moves ln f; twice the larger one is a bound
+      const int rise = ((__double2hiint((double)moves * lnf) & 0x7fffffff) >> 20) + 1;
+      grid = !frozen && max(high + 1, rise) + 1 - low <= 53 && low > 0;
+    }
+    // ln g after n more moves in the same bin: n rounded additions of ln f
+    auto advance = [&](double v, int n) -> double {
+      for (; n > 0 && !frozen; --n) v = __dadd_rn(v, lnf);
+      return v;
+    };
+    const bool wild = !(fabs(lnf) < 1e6);
+    double entry = order_value(lng_s[r]);     // ln g of the bin at move e_in; grid: drawn back to the batch's first move
     uint32_t acc_prev = 0;
     long long n_acc = 0, n_rec = 0;
     for (int b = 0; b < nb; ++b) {
       const int cur = b & 1;
       named_sync(kBarReady + cur);
       const int nvalid = bad ? 0 : (int)(moves - (long long)b * 32 < 32 ? moves - (long long)b * 32 : 32);
-      uint32_t acc_cur = 0;
-      const int4* R4 = reinterpret_cast<const int4*>(rec + cur * 32);
-      // records are read one move ahead, before the stores of the current move
-      int4 nxt[kWords];
-      if (nvalid > 0) {
-#pragma unroll
-        for (int q = 0; q < kWords; ++q) nxt[q] = R4[q];
-      }
-      for (int k = 0; k < nvalid; ++k) {
-        TrajRec r;
-        memcpy(&r, nxt, sizeof r);
-        if (k + 1 < nvalid) {
-#pragma unroll
-          for (int q = 0; q < kWords; ++q) nxt[q] = R4[(k + 1) * kWords + q];
-        }
-        const uint32_t need = (r.cprev & acc_prev) | (r.ccur & acc_cur);
-        const int site = r.site;
-        double dE = r.dE;
-        if (need) {
-          __syncwarp();
-          int X, Y, Z;
-          bcc_coords(site, L, a.geo.divL, X, Y, Z);
-          double dn = 0.0;
-          if (lane == 0)
-            dn = (double)delta_energy<true>(a, off_s, J_s, lat, site, X, Y, Z, r.nx, r.ny, r.nz, 0, 1, 1u);
-          dE = __shfl_sync(kFullMask, dn, 0);
-          ++n_rec;
-        }
-        const double Ep = __dadd_rn(E, dE);
-        const int bp = bin_fp64(Ep, a.win);
-        const int rel = bp - wlo;
-        bool acc = false;
-        if ((unsigned)rel < (unsigned)W) {
-          const double lngp = (bp == bcur) ? lng_cur : lng_s[rel];
-          const double d = __dsub_rn(lng_cur, lngp);
-          acc = (d >= 0.0) || (r.u < exp_fp64(d, a.ex));
-          if (acc) {
-            if (bp != bcur) {
-              lng_s[bcur - wlo] = lng_cur;
-              H_s[bcur - wlo] = h_cur;
-              lng_cur = lngp;
-              h_cur = H_s[rel];
-              bcur = bp;
-            }
-            E = Ep;
+      const bool valid = lane < nvalid;
+      const TrajBatch& B = rec[cur];
+      const int4 move = B.move[lane], marks = B.marks[lane];
+      const int site = move.x;
+      const float lu = __int_as_float(move.z);
+      double dE = B.dE[lane];
+      const double nx = B.nx[lane], ny = B.ny[lane], nz = B.nz[lane];
+      int dq = move.w;
+      const uint32_t cc = (uint32_t)marks.y;
+      bool stale = valid && ((uint32_t)marks.x & acc_prev) != 0u;       // dE is of an older lattice
+      // dE of moves `todo` again, on the lattice as it is
+      auto refresh = [&](uint32_t todo) {
+        __syncwarp();
+        for (; todo; todo &= todo - 1u) {
+          const int k = __ffs(todo) - 1;
+          const int4 mk = B.move[k];
+          const double v = traj_again<NSH>(lat, off_s, J_s, mk.x, (uint32_t)mk.y, B.nx[k], B.ny[k], B.nz[k], L, lane);
+          if (lane == k) {
+            dE = v;
+            dq = traj_units(v, bin_units);
+            stale = false;
           }
         }
-        if (acc) {
-          acc_cur |= 1u << k;
-          ++n_acc;
-          if (lane == 0) lat.set(site, r.nx, r.ny, r.nz);
+        __syncwarp();
+      };
+      refresh(__ballot_sync(kFullMask, stale && cc == 0u));    // (the others may go stale again before their turn)
+      // position of E above the bottom of bin r0, 2^-24 bins; lost: nowhere near (the state was set from outside)
+      int at, r0;
+      bool lost;
+      auto locate = [&]() {
+        r0 = r;
+        const double q = (E - a.win.e_min) * bin_units - (double)(wlo + r) * 16777216.0;
+        lost = !(fabs(q) < 16.0 * kBin);
+        at = lost ? 0 : __double2int_rn(q);
+      };
+      locate();
+      // ln g(target) up to klo: accepted; from khi: rejected; between, or where |ln g| is beyond what they are good
+      // for: open
+      const double from_lo = lane_lnf - (double)lu - kTol, from_hi = lane_lnf - (double)lu + kTol;
+      long long klo, khi;
+      bool far;
+      auto thresholds = [&](double L0) {      // L0: ln g of the bin drawn back to the batch's first move
+        far = (__double2hiint(L0) & 0x7fffffff) >= 0x41cdcd65 || wild || lu > 0.0f;      // 1e9
+        klo = order_key(L0 + from_lo);
+        khi = order_key(L0 + from_hi);
+      };
+      thresholds(entry);
+      // ln g of the bin at move k
+      int e_in = 0;
+      auto lng_at = [&](int k) -> double {
+        if (grid) return entry + (double)k * lnf;
+        return advance(entry, k - e_in);
+      };
+      uint32_t acc_cur = 0;
+      int rb = r;                             // bin after this lane's move
+      bool live = valid;
+      while (true) {
+        const int pos = at + dq, db = pos >> 24;
+        const int rel = r0 + db;
+        const int fr = pos & (kBin - 1);
+        const bool inw = (unsigned)rel < (unsigned)W;
+        const long long lt = lng_s[min((unsigned)rel, (unsigned)W - 1u)];
+        const bool sure = !stale && !far && !lost && (unsigned)(dq + kFarUnits - 1) < 2u * kFarUnits - 1u &&
+                          (unsigned)(fr - kEdge) < (unsigned)(kBin - 2 * kEdge);
+        const bool same_bin = rel == r;
+        const bool yes = inw && (same_bin || lt <= klo);
+        const bool no = !inw || (!same_bin && lt >= khi);
+        const double cand = order_value(lt) - lane_lnf;
+        const uint32_t code = (uint32_t)(dq + 4 * kBin);
+        const uint32_t m = __reduce_min_sync(
+            kFullMask, live && !(sure && no) ? lane_key | (sure && yes && code < kRare ? code : kRare) : kNoKey);
+        const int e = (int)(m >> 27);
+        live = live && lane > e;
+        const double E_step = __shfl_sync(kFullMask, dE, e);
+        int re, seen;                         // bin of the move; the bin that the integers gave it
+        if ((m & kPayload) < kRare) {
+          at += (int)(m & kPayload) - 4 * kBin;
+          re = seen = r0 + (at >> 24);
+        } else {
+          if (m == kNoKey) break;             // every move left is rejected
+          // stale, uncertain or long
+          if (__shfl_sync(kFullMask, (int)stale, e)) {
+            refresh(1u << e);
+            live = live || (lane == e);
+            continue;
+          }
+          const int de = __shfl_sync(kFullMask, dq, e);
+          re = seen = __shfl_sync(kFullMask, rel, e);
+          if (__shfl_sync(kFullMask, (int)!(sure && yes), e)) {
+            // the specified operations
+            re = bin_fp64(__dadd_rn(E, E_step), a.win) - wlo;
+            bool accept = false;
+            if ((unsigned)re < (unsigned)W) {
+              const double L = lng_at(e);
+              const double d = __dsub_rn(L, re == r ? L : order_value(lng_s[re]));
+              accept = (d >= 0.0) || (B.u[e] < exp_fp64(d, a.ex));
+            }
+            if (!accept) continue;
+          }
+          at += de;
         }
-        if (!frozen) {
-          lng_cur = __dadd_rn(lng_cur, lnf);
-          ++h_cur;
+        if (re != r) {
+          double L0 = __shfl_sync(kFullMask, cand, e);
+          if (seen != re) L0 = order_value(lng_s[re]) - __shfl_sync(kFullMask, lane_lnf, e);
+          thresholds(L0);
+          if (grid) {
+            lng_s[r] = order_key(entry + __shfl_sync(kFullMask, lane_lnf, e));
+            entry = L0;
+          } else {
+            lng_s[r] = traj_key(advance(entry, e - e_in));
+            entry = order_value(lng_s[re]);
+          }
+          e_in = e;
+          r = re;
+          rb = lane >= e ? r : rb;
         }
+        E = __dadd_rn(E, E_step);
+        acc_cur |= 1u << e;
+        if (lane == e) lat.set(site, nx, ny, nz);
+        stale = stale || ((cc >> e) & 1u) != 0u;
+        if (lost || !((unsigned)(at + 16 * kBin) < 32u * kBin)) locate();   // positions are relative to bin r0
       }
+      entry = lng_at(nvalid);
+      if (!frozen && valid) atomicAdd(&H_s[rb], 1u);
+      n_rec += __popc(__ballot_sync(kFullMask, valid && (((uint32_t)marks.z & acc_prev) | ((uint32_t)marks.w & acc_cur)) != 0u));
+      n_acc += __popc(acc_cur);
       acc_prev = acc_cur;
       __syncwarp();
       named_arrive(kBarDone + cur);
     }
     if (lane == 0 && !bad) {
       a.st.E[slot] = E;
-      a.st.bin[slot] = bcur;
-      lng_s[bcur - wlo] = lng_cur;
-      H_s[bcur - wlo] = h_cur;
+      a.st.bin[slot] = r + wlo;
+      lng_s[r] = traj_key(entry);
       a.st.steps[slot] = t0 + moves;
       a.st.accepts[slot] += n_acc;
       a.st.recomputes[slot] += n_rec;
@@ -461,7 +645,7 @@ __device__ __forceinline__ void pipe_walk_slot(const WalkerArgs& a, const int sl
       if (lane == 0) atomicExch(a.st.ctrl + 0, kErrOutOfWindow);
       r = 0;                                // no move is made
     }
-    long long A = (long long)lng_s[r];
+    long long A = lng_s[r];
     const long long lane_lnf = (long long)lane * lnf_eff;
     constexpr int kBin = 1 << 24;
     constexpr uint32_t kNoKey = 0xffffffffu;
@@ -592,9 +776,9 @@ __device__ __forceinline__ void pipe_walk_slot(const WalkerArgs& a, const int sl
       // the accepted move e leaves the bin for bin r + db
       auto change_bin = [&](const int e, const int db) {
         const long long el = (long long)e * lnf_eff;
-        lng_s[r] = (Lng)(A + el);
+        lng_s[r] = (A + el);
         r += db;
-        A = (long long)lng_s[r] - el;
+        A = lng_s[r] - el;
         rb = lane > e ? r : rb;
         ++n_chg;
       };
@@ -603,14 +787,14 @@ __device__ __forceinline__ void pipe_walk_slot(const WalkerArgs& a, const int sl
       int lo = 0;
       uint32_t span = 0;
       auto pass = [&]() {
-        const bool up = r + 1 < W && (long long)lng_s[min(r + 1, W - 1)] <= A + Q;
-        const bool down = r > 0 && (long long)lng_s[max(r - 1, 0)] <= A + Q;
+        const bool up = r + 1 < W && lng_s[min(r + 1, W - 1)] <= A + Q;
+        const bool down = r > 0 && lng_s[max(r - 1, 0)] <= A + Q;
         lo = down ? -kBin : 0;
         span = (uint32_t)(kBin + (up ? kBin : 0) - lo);
       };
       // the target bin r + db of move e, looked up
       auto admits = [&](const int e, const int db) -> bool {
-        return (unsigned)(r + db) < (unsigned)W && (long long)lng_s[r + db] <= A + shfl_ll(Q, e);
+        return (unsigned)(r + db) < (unsigned)W && lng_s[r + db] <= A + shfl_ll(Q, e);
       };
       if (path == kSequential && __popc(touched) >= kDense) {
         // Many moves touch a later one (small lattices): every round pushes, without asking.  Measured,
@@ -622,7 +806,7 @@ __device__ __forceinline__ void pipe_walk_slot(const WalkerArgs& a, const int sl
         bool live = valid;
         while (true) {
           const int pos = frac + dq, rel = r + (pos >> 24);
-          const long long lt = (long long)lng_s[min((unsigned)rel, (unsigned)W - 1u)];
+          const long long lt = lng_s[min((unsigned)rel, (unsigned)W - 1u)];
           const bool plain = (unsigned)(dq + 4 * kBin - 1) < 8u * kBin - 1u && dq != -1;
           const uint32_t key = lane_key | (plain ? (uint32_t)dq & kPayload : kRare);
           // ln g of the walker's own bin in the table is at most its present value, so a move that
@@ -636,7 +820,7 @@ __device__ __forceinline__ void pipe_walk_slot(const WalkerArgs& a, const int sl
             if (m == kNoKey) break;        // every move left is rejected
             pe = __shfl_sync(kFullMask, pos, e);
           }
-          lng_s[r] = (Lng)(A + (long long)e * lnf_eff);
+          lng_s[r] = (A + (long long)e * lnf_eff);
           n_chg += (pe >> 24) != 0 ? 1 : 0;
           r += pe >> 24;
           frac = pe & (kBin - 1);
@@ -663,7 +847,7 @@ __device__ __forceinline__ void pipe_walk_slot(const WalkerArgs& a, const int sl
         auto look = [&]() {
           pos = at + dq;
           rel = r0 + (pos >> 24);
-          lt = (long long)lng_s[min((unsigned)rel, (unsigned)W - 1u)];
+          lt = lng_s[min((unsigned)rel, (unsigned)W - 1u)];
         };
         look();
         bool away = false;
@@ -676,14 +860,14 @@ __device__ __forceinline__ void pipe_walk_slot(const WalkerArgs& a, const int sl
           const long long A2 = shfl_ll(rel == r ? A : lt - lane_lnf, e);   // ln g after the move, less e ln f
           const bool rare = (m & kPayload) == kRare || m == kNoKey || away;
           const int at2 = at + ((int)(m << 5) >> 5);
-          if (!rare) lng_s[r] = (Lng)(A + (long long)e * lnf_eff);
+          if (!rare) lng_s[r] = (A + (long long)e * lnf_eff);
           const int pos2 = at2 + dq, rel2 = r0 + (pos2 >> 24);
-          const long long lt2 = (long long)lng_s[min((unsigned)rel2, (unsigned)W - 1u)];
+          const long long lt2 = lng_s[min((unsigned)rel2, (unsigned)W - 1u)];
           int rn;
           if (rare) {
             if (m == kNoKey) break;        // every move left is rejected
             const int pe = __shfl_sync(kFullMask, pos, e);
-            lng_s[r] = (Lng)(A + (long long)e * lnf_eff);
+            lng_s[r] = (A + (long long)e * lnf_eff);
             r0 += pe >> 24;
             at = pe & (kBin - 1);
             rn = r0;
@@ -873,7 +1057,7 @@ __device__ __forceinline__ void pipe_walk_slot(const WalkerArgs& a, const int sl
     const unsigned corrected = __reduce_add_sync(kFullMask, n_rec);
     if (lane == 0 && !bad) {
       a.st.efx[slot] = ((long long)(r + wlo) << 32) | (long long)(((uint32_t)frac << 8) | frac_low);
-      lng_s[r] = (Lng)A;
+      lng_s[r] = A;
       a.st.steps[slot] = t0 + moves;
       a.st.accepts[slot] += n_acc;
       a.st.recomputes[slot] += corrected;
@@ -888,9 +1072,9 @@ __device__ __forceinline__ void pipe_walk_slot(const WalkerArgs& a, const int sl
   if constexpr (kSmem) copy_lattice(glat, lat, N, tid, nt);
   for (int w = tid; w < W; w += nt) {
     if constexpr (kTraj)
-      a.st.lng[lbase + w] = (double)lng_s[w];
+      a.st.lng[lbase + w] = order_value(lng_s[w]);
     else
-      a.st.lng_fx[lbase + w] = (long long)lng_s[w];
+      a.st.lng_fx[lbase + w] = lng_s[w];
     a.st.H[lbase + w] = H_s[w];
   }
   if constexpr (kTraj) {       // production: energy_update_kernel, after the walk
