@@ -297,12 +297,12 @@ __device__ __forceinline__ float u24_sym(uint32_t x) {
 }
 
 __device__ __forceinline__ void draw_prod(uint2 key, unsigned long long t, bool init, int N, int& site,
-                                          long long& lu, float& nx, float& ny, float& nz) {
+                                          float& ln_u, float& nx, float& ny, float& nz) {
   const uint32_t lo = (uint32_t)t, hi = (uint32_t)(t >> 32);
   const uint4 x = philox10(make_uint4(lo, hi, init ? 2u : 0u, 0u), key);
   site = (int)__umulhi(x.x, (uint32_t)N);
   const float uf = fmaf(__uint2float_rn(x.y), 0x1.0p-32f, 0x1.0p-33f);   // (0, 1]
-  lu = __float2ll_rn(logf(uf) * 0x1.0p40f);
+  ln_u = logf(uf);
   float a = u24_sym(x.z), b = u24_sym(x.w);
   float q = fmaf(a, a, b * b);
   uint32_t k = 0;
