@@ -261,23 +261,20 @@ __device__ __forceinline__ long long to_units(float dE, double scale, float limi
 // The slots of a lane of a group of G on a bcc lattice, slots sub, sub + G, .. of the canonical order, held in
 // registers.  The sum of delta_energy, without its loop: the loads of all slots are in flight together.  (The
 // initial drive of bcc L = 12, 2 shells, 64 walkers, one lane per move: 640 us with the loop, 370 us so.)
-template <int kG, int kSlots>
+template <int kG, int kSlots, bool kHeld>     // kHeld: in registers, else read from shared memory for each move
 struct LaneSlots {
-  static constexpr bool kPacked = kSlots > 8;   // registers: many slots stay packed and leave J in shared memory
-  int dx[kPacked ? 1 : kSlots], dy[kPacked ? 1 : kSlots], dz[kPacked ? 1 : kSlots];
-  uint32_t off[kPacked ? kSlots : 1];
-  float J[kPacked ? 1 : kSlots];
-  const float* J_at;                            // J of slot q: J_at[kG q]
+  int dx[kHeld ? kSlots : 1], dy[kHeld ? kSlots : 1], dz[kHeld ? kSlots : 1];
+  float J[kHeld ? kSlots : 1];
+  const uint32_t* off_at;                       // slot q: off_at[kG q], J_at[kG q] (of kMaxSlotsPerSite entries)
+  const float* J_at;
   uint32_t have = 0, opens = 0;               // slots that exist; that begin another shell
-  __device__ __forceinline__ LaneSlots(const uint32_t* off_s, const float* J_s, int sub, int z) : J_at(J_s + sub) {
+  __device__ __forceinline__ LaneSlots(const uint32_t* off_s, const float* J_s, int sub, int z) : off_at(off_s + (sub < z ? sub : 0)), J_at(J_s + sub) {
     uint32_t shell = 0xffffffffu;
 #pragma unroll
     for (int q = 0; q < kSlots; ++q) {
       const int j = sub + q * kG;
       const uint32_t o = off_s[j < z ? j : 0];
-      if constexpr (kPacked) {
-        off[q] = o;
-      } else {
+      if constexpr (kHeld) {
         unpack_offset(o, dx[q], dy[q], dz[q]);
         J[q] = J_s[j < z ? j : 0];
       }
@@ -294,12 +291,12 @@ struct LaneSlots {
 #pragma unroll
     for (int q = 0; q < kSlots; ++q) {
       int ox, oy, oz;
-      if constexpr (kPacked) {
-        unpack_offset(off[q], ox, oy, oz);
-      } else {
+      if constexpr (kHeld) {
         ox = dx[q];
         oy = dy[q];
         oz = dz[q];
+      } else {
+        unpack_offset(((have >> q) & 1u) != 0u ? off_at[kG * q] : off_at[0], ox, oy, oz);
       }
       lat.get(bcc_offset_site((int)(place & 1023u), (int)((place >> 10) & 1023u), (int)(place >> 20), ox, oy, oz, L), vx[q],
               vy[q], vz[q]);
@@ -317,11 +314,10 @@ struct LaneSlots {
       tx = open ? 0.0f : tx;
       ty = open ? 0.0f : ty;
       tz = open ? 0.0f : tz;
-      // (a slot that opens a shell exists, so J_at stays within the table)
-      if constexpr (kPacked)
-        Jc = open ? J_at[kG * q] : Jc;
-      else
+      if constexpr (kHeld)
         Jc = open ? J[q] : Jc;
+      else
+        Jc = open ? J_at[kG * q] : Jc;
       const float sx = tx + vx[q], sy = ty + vy[q], sz = tz + vz[q];
       tx = add ? sx : tx;
       ty = add ? sy : ty;
@@ -340,8 +336,8 @@ struct LaneSlots {
     return -fmaf(dz0, hz, fmaf(dy0, hy, dx0 * hx));
   }
 };
-template <int kG>
-struct LaneSlots<kG, 0> {
+template <int kG, bool kHeld>
+struct LaneSlots<kG, 0, kHeld> {
   __device__ __forceinline__ LaneSlots(const uint32_t*, const float*, int, int) {}
 };
 
@@ -378,7 +374,7 @@ __device__ __forceinline__ void walk_units(const WalkerArgs& a, int slot, int wl
   long long n_acc = 0, n_rec = 0;
   const long long g_lnf = (long long)g * lnf;
   const float limit = (float)(0x1.0p49 / a.win.dq_scale64);
-  const LaneSlots<kG, kSlots> slots(off_s, J_s, sub, a.geo.z);
+  const LaneSlots<kG, kSlots, !kInit || kSlots <= 2> slots(off_s, J_s, sub, a.geo.z);
 
   for (int c = 0;; ++c) {
     pair_sync(kBarDrawn);
@@ -480,8 +476,8 @@ __device__ __forceinline__ void walk_units(const WalkerArgs& a, int slot, int wl
   __syncwarp();
 }
 
-template <bool kTraj, bool kSmem>
-__global__ void __launch_bounds__(kWalkerThreads) walker_kernel(const WalkerArgs a) {
+template <bool kTraj, bool kSmem, bool kInit, int kG, int kSlots>
+__global__ void __launch_bounds__(kWalkerThreads, kTraj ? 1 : kInit ? 7 : kSlots > 2 ? 4 : 6) walker_kernel(const WalkerArgs a) {
   using Real = typename Mode<kTraj>::Real;
   using Lng = typename Mode<kTraj>::Lng;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -529,33 +525,9 @@ __global__ void __launch_bounds__(kWalkerThreads) walker_kernel(const WalkerArgs
   if constexpr (kTraj) {
     if (tid < 32) walk(a, slot, wlo, lng_s, H_s, off_s, J_s, lat);
   } else {
-    // bcc: lanes per move and slots per lane, for the couplings of 1 to 4 shells (8, 14, 26, 50 slots) and the
-    // groups that the size rule picks for them; one lane per move only for the initial drive, as the pipelined
-    // walker walks such lattices.  Other groups, and lattices given as tables, run the loop.
-    const int n = a.geo.kind == 0 ? (a.geo.z + a.G - 1) / a.G : 99;
-    auto go = [&](auto init) {
-      constexpr bool kInit = decltype(init)::value;
-      if (a.G == 16 && n <= 4)
-        walk_units<kInit, 16, 4>(a, slot, wlo, lng_s, H_s, off_s, J_s, lat, draws);
-      else if (a.G == 8 && n <= 2)
-        walk_units<kInit, 8, 2>(a, slot, wlo, lng_s, H_s, off_s, J_s, lat, draws);
-      else if (a.G == 8 && n <= 7)
-        walk_units<kInit, 8, 7>(a, slot, wlo, lng_s, H_s, off_s, J_s, lat, draws);
-      else if (a.G == 4 && n <= 7)
-        walk_units<kInit, 4, 7>(a, slot, wlo, lng_s, H_s, off_s, J_s, lat, draws);
-      else if (kInit && a.G == 1 && n <= 14)
-        walk_units<kInit, kInit ? 1 : 0, kInit ? 14 : 0>(a, slot, wlo, lng_s, H_s, off_s, J_s, lat, draws);
-      else if (kInit && a.G == 1 && n <= 26)
-        walk_units<kInit, kInit ? 1 : 0, kInit ? 26 : 0>(a, slot, wlo, lng_s, H_s, off_s, J_s, lat, draws);
-      else
-        walk_units<kInit, 0, 0>(a, slot, wlo, lng_s, H_s, off_s, J_s, lat, draws);
-    };
-    if (tid < 32) {
-      if (a.init)
-        go(std::true_type{});
-      else
-        go(std::false_type{});
-    } else if (tid < 64)
+    if (tid < 32)
+      walk_units<kInit, kG, kSlots>(a, slot, wlo, lng_s, H_s, off_s, J_s, lat, draws);
+    else if (tid < 64)
       draw_moves(a, slot, draws);
   }
   __syncthreads();
@@ -637,23 +609,42 @@ size_t walker_smem_bytes(bool traj, bool smem_lattice, int N, int W) {
   return bytes;
 }
 
+template <bool kTraj, bool kSmem, bool kInit, int kG, int kSlots>
+static cudaError_t launch_walker_kernel(const WalkerArgs& a, int n_slots, size_t smem, cudaStream_t stream) {
+  const auto kernel = walker_kernel<kTraj, kSmem, kInit, kG, kSlots>;
+  const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  kernel<<<n_slots, kWalkerThreads, smem, stream>>>(a);
+  return cudaGetLastError();
+}
+
+template <bool kSmem, bool kInit>
+static cudaError_t launch_units(const WalkerArgs& a, int n_slots, size_t smem, cudaStream_t stream) {
+  // bcc: lanes per move and slots per lane, for the couplings of 1 to 4 shells (8, 14, 26, 50 slots) and the
+  // groups that the size rule picks for them; one lane per move only for the initial drive, as the pipelined
+  // walker walks such lattices.  Other groups, and lattices given as tables, run the loop.
+  const int n = a.geo.kind == 0 ? (a.geo.z + a.G - 1) / a.G : 99;
+  if (a.G == 16 && n <= 4) return launch_walker_kernel<false, kSmem, kInit, 16, 4>(a, n_slots, smem, stream);
+  if (a.G == 8 && n <= 2) return launch_walker_kernel<false, kSmem, kInit, 8, 2>(a, n_slots, smem, stream);
+  if (a.G == 8 && n <= 7) return launch_walker_kernel<false, kSmem, kInit, 8, 7>(a, n_slots, smem, stream);
+  if (a.G == 4 && n <= 7) return launch_walker_kernel<false, kSmem, kInit, 4, 7>(a, n_slots, smem, stream);
+  if constexpr (kInit) {
+    if (a.G == 1 && n <= 14) return launch_walker_kernel<false, kSmem, true, 1, 14>(a, n_slots, smem, stream);
+    if (a.G == 1 && n <= 26) return launch_walker_kernel<false, kSmem, true, 1, 26>(a, n_slots, smem, stream);
+  }
+  return launch_walker_kernel<false, kSmem, kInit, 0, 0>(a, n_slots, smem, stream);
+}
+
 cudaError_t launch_walkers(const WalkerArgs& a, int n_slots, bool traj, bool smem_lattice, size_t smem,
                            cudaStream_t stream) {
-  cudaError_t e = cudaSuccess;
-  if (traj && smem_lattice) {
-    e = cudaFuncSetAttribute(walker_kernel<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e == cudaSuccess) walker_kernel<true, true><<<n_slots, kWalkerThreads, smem, stream>>>(a);
-  } else if (traj) {
-    e = cudaFuncSetAttribute(walker_kernel<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e == cudaSuccess) walker_kernel<true, false><<<n_slots, kWalkerThreads, smem, stream>>>(a);
-  } else if (smem_lattice) {
-    e = cudaFuncSetAttribute(walker_kernel<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e == cudaSuccess) walker_kernel<false, true><<<n_slots, kWalkerThreads, smem, stream>>>(a);
-  } else {
-    e = cudaFuncSetAttribute(walker_kernel<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e == cudaSuccess) walker_kernel<false, false><<<n_slots, kWalkerThreads, smem, stream>>>(a);
-  }
-  if (e == cudaSuccess) e = cudaGetLastError();
+  cudaError_t e;
+  if (traj)
+    e = smem_lattice ? launch_walker_kernel<true, true, false, 0, 0>(a, n_slots, smem, stream)
+                     : launch_walker_kernel<true, false, false, 0, 0>(a, n_slots, smem, stream);
+  else if (a.init)
+    e = smem_lattice ? launch_units<true, true>(a, n_slots, smem, stream) : launch_units<false, true>(a, n_slots, smem, stream);
+  else
+    e = smem_lattice ? launch_units<true, false>(a, n_slots, smem, stream) : launch_units<false, false>(a, n_slots, smem, stream);
   if (e == cudaSuccess && a.recompute && !a.init && !traj && a.geo.kind == 0)
     e = launch_energy_update(a, n_slots, stream);
   return e;
