@@ -260,7 +260,7 @@ __device__ __forceinline__ long long to_units(float dE, double scale, float limi
 
 // The slots of a lane of a group of G on a bcc lattice, slots sub, sub + G, .. of the canonical order, held in
 // registers.  The sum of delta_energy, without its loop: the loads of all slots are in flight together.  (The
-// initial drive of bcc L = 12, 2 shells, 64 walkers, one lane per move: 640 us with the loop, 370 us so.)
+// initial drive of bcc L = 12, 2 shells, 64 walkers, one lane per move: 640 us with the loop, 470 us so.)
 template <int kG, int kSlots, bool kHeld>     // kHeld: in registers, else read from shared memory for each move
 struct LaneSlots {
   int dx[kHeld ? kSlots : 1], dy[kHeld ? kSlots : 1], dz[kHeld ? kSlots : 1];
@@ -399,13 +399,19 @@ __device__ __forceinline__ void walk_units(const WalkerArgs& a, int slot, int wl
       while (true) {
         if (again) {
           __syncwarp();
-          float dE;
-          if constexpr (kSlots > 0)
-            dE = slots.delta(lat, site, place, nx, ny, nz, a.geo.L);
-          else
+          const bool mine = (conf & again) != 0u || acc_mask == 0u;
+          float dE = 0.0f;
+          if constexpr (kSlots > 0) {
+            // (one lane per move and a lattice in global memory: only the moves in question load their neighbours)
+            if (kG > 1 || std::is_same<Lat, CodePlanes>::value || mine) dE = slots.delta(lat, site, place, nx, ny, nz, a.geo.L);
+          } else if (G == 1) {
+            if (mine) dE = delta_energy<false>(a, off_s, J_s, lat, site, X, Y, Z, nx, ny, nz, 0, 1, 0u);
+            __syncwarp();
+          } else {
             dE = delta_energy<false>(a, off_s, J_s, lat, site, X, Y, Z, nx, ny, nz, sub, G, kFullMask);
+          }
           const long long units = to_units(dE, a.win.dq_scale64, limit);
-          dq = (conf & again) != 0u || acc_mask == 0u ? units : dq;
+          dq = mine ? units : dq;
           again = 0u;
         }
         const long long Ep = Efx + dq;
@@ -476,8 +482,12 @@ __device__ __forceinline__ void walk_units(const WalkerArgs& a, int slot, int wl
   __syncwarp();
 }
 
+// Walkers that an SM is to hold (production): seven in the initial drive, which starts all of them at once, and with
+// up to two slots per lane (2048 walkers of bcc L = 4: 586 us per 1000 moves, 733 us with six); four with more slots,
+// held in registers (512 walkers of bcc L = 8: 264 us; 311 us with six and the slots in shared memory).
 template <bool kTraj, bool kSmem, bool kInit, int kG, int kSlots>
-__global__ void __launch_bounds__(kWalkerThreads, kTraj ? 1 : kInit ? 7 : kSlots > 2 ? 4 : 6) walker_kernel(const WalkerArgs a) {
+__global__ void __launch_bounds__(kWalkerThreads, kTraj ? 1 : kInit || kSlots <= 2 ? 7 : 4)
+    walker_kernel(const WalkerArgs a) {
   using Real = typename Mode<kTraj>::Real;
   using Lng = typename Mode<kTraj>::Lng;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -630,7 +640,6 @@ static cudaError_t launch_units(const WalkerArgs& a, int n_slots, size_t smem, c
   if (a.G == 4 && n <= 7) return launch_walker_kernel<false, kSmem, kInit, 4, 7>(a, n_slots, smem, stream);
   if constexpr (kInit) {
     if (a.G == 1 && n <= 14) return launch_walker_kernel<false, kSmem, true, 1, 14>(a, n_slots, smem, stream);
-    if (a.G == 1 && n <= 26) return launch_walker_kernel<false, kSmem, true, 1, 26>(a, n_slots, smem, stream);
   }
   return launch_walker_kernel<false, kSmem, kInit, 0, 0>(a, n_slots, smem, stream);
 }
