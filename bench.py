@@ -465,7 +465,8 @@ def run_batch64(args):
                        "l2": "flushed between steps (256 MB write)", "graph": True,
                        "tuning": tune, "batch": info, "setup_s": setup_s},
             "e2e": {"value": e2e_value, "unit": UNIT, "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h},
-            "gpu_launches": args.steps * I * 3,
+            # walker, exchange, flatness per interval; the energy recomputation every eighth
+            "gpu_launches": args.steps * I * 3 + args.steps * I // 8,
             "clocks": clk,
         }
         print(json.dumps(line), flush=True)
@@ -821,7 +822,8 @@ def main():
                          "sms_used": min(S, torch.cuda.get_device_properties(dev).multi_processor_count),
                          "peak_source": peak_source},
             "e2e": {"value": e2e_value, "unit": UNIT, "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h},
-            "gpu_launches": args.steps * (3 * I + 2),
+            # walker, exchange, flatness per interval; the energy recomputation every eighth; three per merge
+            "gpu_launches": args.steps * (3 * I + 3) + args.steps * I // 8,
             "clocks": clk,
         }
         if cpu is not None:
