@@ -643,10 +643,10 @@ static rewl_status create_impl(const rewl_lattice* lat, const rewl_couplings* cp
   if (g.kind == 0 && h->G == 1 && max_dE < 100.0 * h->dE) {
     int own_full = 256;
     while (own_full < h->N && own_full < 8192) own_full *= 2;
-    const size_t base = walker_pipe_smem_bytes(h->traj, true, h->N, h->W, 0);
-    if (base + 1024 + 256 * 8 <= (size_t)max_smem) {
+    const size_t limit = (size_t)max_smem - 1024;
+    if (walker_pipe_fits(h->traj, true, h->N, h->W, 256, limit)) {
       int e = own_full;
-      while (e > 256 && base + 1024 + 8 * (size_t)e > (size_t)max_smem) e /= 2;
+      while (e > 256 && !walker_pipe_fits(h->traj, true, h->N, h->W, e, limit)) e /= 2;
       h->own_entries = e;
       h->pipe_smem_lattice = true;
     } else {
@@ -655,8 +655,9 @@ static rewl_status create_impl(const rewl_lattice* lat, const rewl_couplings* cp
       h->own_entries = std::min(own_full, kGlobalLatticeOwnEntries);
       h->pipe_smem_lattice = false;
     }
+    h->pipe = walker_pipe_fits(h->traj, h->pipe_smem_lattice, h->N, h->W, h->own_entries, limit);
+    if (h->pipe) h->own_entries = walker_pipe_table(h->traj, h->pipe_smem_lattice, h->N, h->W, h->own_entries, limit);
     h->pipe_smem_bytes = walker_pipe_smem_bytes(h->traj, h->pipe_smem_lattice, h->N, h->W, h->own_entries);
-    h->pipe = h->pipe_smem_bytes + 1024 <= (size_t)max_smem;
   }
 
   const size_t S = h->S, W = h->W, N = h->N, X = (size_t)std::max(h->h - 1, 1);
@@ -924,8 +925,8 @@ rewl_status rewl_autotune(rewl_handle* h, int64_t trial_moves, int32_t* entries_
   // walker per SM.
   std::vector<int> cands;
   for (int c = own_full; c >= 512; c /= 2)
-    if (walker_pipe_smem_bytes(h->traj, h->pipe_smem_lattice, h->N, h->W, c) + 1024 <= (size_t)max_smem)
-      cands.push_back(c);
+    if (walker_pipe_fits(h->traj, h->pipe_smem_lattice, h->N, h->W, c, (size_t)max_smem - 1024))
+      cands.push_back(walker_pipe_table(h->traj, h->pipe_smem_lattice, h->N, h->W, c, (size_t)max_smem - 1024));
   if (cands.size() < 2) {   // nothing to choose between: no trial, no move
     cudaEventDestroy(e0);
     if (e1) cudaEventDestroy(e1);

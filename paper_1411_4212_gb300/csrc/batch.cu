@@ -92,10 +92,11 @@ int own_full_entries(int N, bool smem_lattice, int own_cap) {
   return e;
 }
 
-// Largest owner table (power of two, 256 .. own_full_entries) that fits `cap` bytes; 0 if none.
+// Largest owner table (power of two, 256 .. own_full_entries, or what walker_pipe_table makes of it) that fits `cap`
+// bytes; 0 if none.
 int fit_owner(bool traj, bool smem_lattice, int N, int W, size_t cap, int own_cap) {
   for (int e = own_full_entries(N, smem_lattice, own_cap); e >= 256; e /= 2)
-    if (walker_pipe_smem_bytes(traj, smem_lattice, N, W, e) <= cap) return e;
+    if (walker_pipe_fits(traj, smem_lattice, N, W, e, cap)) return walker_pipe_table(traj, smem_lattice, N, W, e, cap);
   return 0;
 }
 
@@ -110,6 +111,7 @@ rewl_status apply_tuning(rewl_batch* b, int workers, int smem_max_n, int own_cap
   const size_t cap = (usable / (size_t)workers) & ~(size_t)15;
   const int n = (int)b->jobs.size();
   std::vector<char> in_smem(n, 0);
+  std::vector<int> table(n, 0);
   size_t arena = 0;
   for (int j = 0; j < n; ++j) {
     const JobView& v = b->view[j];
@@ -118,8 +120,8 @@ rewl_status apply_tuning(rewl_batch* b, int workers, int smem_max_n, int own_cap
       return bfail(b, REWL_EINVAL, "window tables of job " + std::to_string(j) + " do not fit the arena");
     in_smem[j] = s;
     // the smallest arena that still holds this job with its full owner table, else the cap
-    const int e = fit_owner(b->traj, s, v.N, v.W, cap, own_cap);
-    arena = std::max(arena, walker_pipe_smem_bytes(b->traj, s, v.N, v.W, e));
+    table[j] = fit_owner(b->traj, s, v.N, v.W, cap, own_cap);
+    arena = std::max(arena, walker_pipe_smem_bytes(b->traj, s, v.N, v.W, table[j]));
   }
   arena = (arena + 15) & ~(size_t)15;
   int bps = 0;
@@ -135,8 +137,7 @@ rewl_status apply_tuning(rewl_batch* b, int workers, int smem_max_n, int own_cap
     const JobView& v = b->view[j];
     WalkerArgs& a = b->wargs[j];
     a = job_walker_args(b->jobs[j], b->moves, 0);
-    const int e = fit_owner(b->traj, in_smem[j] != 0, v.N, v.W, arena, own_cap);
-    a.own_mask = e - 1;
+    a.own_mask = table[j] - 1;
     a.smem_lattice = in_smem[j];
     b->n_smem_jobs += in_smem[j];
   }

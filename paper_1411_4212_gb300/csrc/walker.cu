@@ -189,7 +189,7 @@ struct DrawBatch {
   uint32_t place[32];    // bcc: half-unit coordinates X | Y << 10 | Z << 20; else the site
   float ln_u[32];
   uint32_t conf[32];     // earlier moves of the batch of K on the same site or a neighbour of it
-  int last;              // chunk in which the walk ended
+  long long last;        // chunk in which the walk ended
 };
 constexpr int kBarDrawn = 1, kBarTaken = 2;   // named barriers of warps 0 and 1
 __device__ __forceinline__ void pair_sync(int id) { asm volatile("bar.sync %0, 64;" ::"r"(id) : "memory"); }
@@ -204,10 +204,10 @@ __device__ __forceinline__ void draw_moves(const WalkerArgs& a, int slot, DrawBa
   const uint2 key = make_uint2((uint32_t)global_slot(a.st, slot), a.key1);
   const unsigned long long t0 = init ? 0ULL : (unsigned long long)a.st.steps[slot];
   const int first = lane / K * K;             // the batch's first move
-  for (int c = 0;; ++c) {
+  for (long long c = 0;; ++c) {
     int site;
     float ln_u, nx, ny, nz;
-    draw_prod(key, t0 + 32ULL * (unsigned)c + (unsigned)lane, init, N, site, ln_u, nx, ny, nz);
+    draw_prod(key, t0 + 32ULL * (unsigned long long)c + (unsigned)lane, init, N, site, ln_u, nx, ny, nz);
     const float2 code = oct_encode(nx, ny, nz);
     uint32_t conf = 0, place = (uint32_t)site;
     if (bcc) {
@@ -235,7 +235,7 @@ __device__ __forceinline__ void draw_moves(const WalkerArgs& a, int slot, DrawBa
     }
     if (c > 0) {
       pair_sync(kBarTaken);                   // chunk c-1
-      if (c > *(volatile int*)&buf.last) return;
+      if (c > *(volatile long long*)&buf.last) return;
     }
     buf.code[lane] = code;
     buf.place[lane] = place;
@@ -376,7 +376,7 @@ __device__ __forceinline__ void walk_units(const WalkerArgs& a, int slot, int wl
   const float limit = (float)(0x1.0p49 / a.win.dq_scale64);
   const LaneSlots<kG, kSlots, !kInit || kSlots <= 2> slots(off_s, J_s, sub, a.geo.z);
 
-  for (int c = 0;; ++c) {
+  for (long long c = 0;; ++c) {
     pair_sync(kBarDrawn);
     for (int first = 0; first < 32 && remaining > 0 && !done; first += K) {
       const int nvalid = (int)(remaining < (long long)K ? remaining : (long long)K);
@@ -462,7 +462,7 @@ __device__ __forceinline__ void walk_units(const WalkerArgs& a, int slot, int wl
       __syncwarp();
     }
     const bool ended = remaining <= 0 || done;
-    if (ended && lane == 0) *(volatile int*)&buf.last = c;
+    if (ended && lane == 0) *(volatile long long*)&buf.last = c;
     __syncwarp();
     pair_arrive(kBarTaken);
     if (ended) break;
@@ -529,7 +529,7 @@ __global__ void __launch_bounds__(kWalkerThreads, kTraj ? 1 : kInit || kSlots <=
     J_s[j] = kTraj ? (Real)a.geo.Jd[j] : (Real)a.geo.Jf[j];
   }
   if constexpr (kSmem) copy_lattice(lat, glat, N, tid, blockDim.x);
-  if (!kTraj && tid == 0) draws.last = 0x7fffffff;
+  if (!kTraj && tid == 0) draws.last = 0x7fffffffffffffffLL;
   __syncthreads();
 
   if constexpr (kTraj) {

@@ -15,6 +15,11 @@ cudaError_t launch_walkers(const WalkerArgs& a, int n_slots, bool traj, bool sme
 
 // Warp-specialised walker (bcc lattices, one lane per trial move, Wang-Landau moves only).
 size_t walker_pipe_smem_bytes(bool traj, bool smem_lattice, int N, int W, int own_entries);
+// Which walkers are pipelined, and which tunings a batch accepts, goes by move records of kRecordBytes (whatever
+// the kernel's own take), so that it does not change with the kernel: walker_pipe_fits.  walker_pipe_table is the
+// conflict table that then fits beside the kernel's records, `own_entries` or half or a quarter of it.
+bool walker_pipe_fits(bool traj, bool smem_lattice, int N, int W, int own_entries, size_t limit);
+int walker_pipe_table(bool traj, bool smem_lattice, int N, int W, int own_entries, size_t limit);
 // a.smem_lattice selects the form: 1 = lattice in shared memory, arguments passed by value (d_args
 // NULL); 0 = lattice in global memory, the kernel reads d_args, a device copy of a (a.moves and
 // a.recompute are passed by value and may differ from the copy).

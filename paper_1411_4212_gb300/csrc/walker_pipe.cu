@@ -1211,6 +1211,17 @@ size_t walker_pipe_smem_bytes(bool traj, bool smem_lattice, int N, int W, int ow
   return bytes;
 }
 
+bool walker_pipe_fits(bool traj, bool smem_lattice, int N, int W, int own_entries, size_t limit) {
+  const size_t kRecordBytes = traj ? 5120 : 6144;
+  return walker_pipe_smem_bytes(traj, smem_lattice, N, W, own_entries) - batch_bytes(traj) + kRecordBytes <= limit;
+}
+
+int walker_pipe_table(bool traj, bool smem_lattice, int N, int W, int own_entries, size_t limit) {
+  static_assert(batch_bytes(true) <= 5120 && batch_bytes(false) <= 6144 + 8 * (256 - 64), "a table of 256 entries gives way");
+  while (own_entries > 64 && walker_pipe_smem_bytes(traj, smem_lattice, N, W, own_entries) > limit) own_entries /= 2;
+  return own_entries;
+}
+
 template <bool kTraj, int NSH>
 static cudaError_t launch_pipe_t(const WalkerArgs& a, const WalkerArgs* d_args, int n_slots, size_t smem,
                                  cudaStream_t stream) {

@@ -60,3 +60,21 @@ def test_a_small_table_beside_a_shared_lattice_changes_nothing():
     _assert_same(_state(alone), _state(batched), "shared lattice, small table")
     alone.close()
     batched.close()
+
+
+@pytest.mark.parametrize("bins,pipelined", [(17000, 1), (17330, 1), (17500, 0)])
+def test_window_tables_up_to_the_shared_memory_limit(bins, pipelined):
+    """bcc L = 24 with one window so wide that its tables fill the shared memory: the widest ones leave the
+    conflict table less room than the rule that admits them counts.  The walk goes by neither."""
+    spec = dict(kind=rw.BCC, L=24, J=J[:2], n_bins=bins, n_windows=1, walkers_per_window=2, overlap=0.0, seed=6,
+                lnf_final=1e-8, exchange_interval=2000, recompute_every=1000, group_size=1)
+    states = []
+    for resolver in (rw.RESOLVER_AUTO, rw.RESOLVER_SEQUENTIAL):
+        g = rw.REWL(resolver=resolver, **spec)
+        assert g.info()["pipelined"] == pipelined
+        g.init_walkers()
+        g.run_intervals(2, stats=False)
+        states.append(_state(g))
+        assert (states[-1]["steps"] == 4000).all()
+        g.close()
+    _assert_same(states[0], states[1], f"{bins} bins")
