@@ -233,6 +233,7 @@ __device__ __forceinline__ void draw_moves(const WalkerArgs& a, int slot, DrawBa
           conf |= n == __shfl_sync(kFullMask, site, first + j) && first + j < lane ? 1u << j : 0u;
       }
     }
+    __syncwarp();                             // (the draws may have diverged)
     if (c > 0) {
       pair_sync(kBarTaken);                   // chunk c-1
       if (c > *(volatile long long*)&buf.last) return;
@@ -377,6 +378,7 @@ __device__ __forceinline__ void walk_units(const WalkerArgs& a, int slot, int wl
   const LaneSlots<kG, kSlots, !kInit || kSlots <= 2> slots(off_s, J_s, sub, a.geo.z);
 
   for (long long c = 0;; ++c) {
+    __syncwarp();
     pair_sync(kBarDrawn);
     for (int first = 0; first < 32 && remaining > 0 && !done; first += K) {
       const int nvalid = (int)(remaining < (long long)K ? remaining : (long long)K);
