@@ -229,10 +229,15 @@ rewl_status order_after_jobs(rewl_batch* b) {
   return REWL_OK;
 }
 
-rewl_status order_jobs_after(rewl_batch* b) {
-  BCUDA(b, cudaEventRecord(b->ev_done, b->stream));
-  for (cudaStream_t s : b->ext) BCUDA(b, cudaStreamWaitEvent(s, b->ev_done, 0));
-  return REWL_OK;
+// The jobs' streams come after everything that the batch has enqueued.  `s` is the outcome of the call that
+// enqueued it and is passed on: a call that ends early has to come through here too, as its jobs may be read or
+// closed next.  Where the streams cannot be ordered, the host waits.
+rewl_status order_jobs_after(rewl_batch* b, rewl_status s) {
+  cudaError_t e = cudaEventRecord(b->ev_done, b->stream);
+  for (size_t i = 0; i < b->ext.size() && e == cudaSuccess; ++i) e = cudaStreamWaitEvent(b->ext[i], b->ev_done, 0);
+  if (e == cudaSuccess) return s;
+  cudaStreamSynchronize(b->stream);
+  return s != REWL_OK ? s : bfail(b, REWL_ECUDA, std::string("order of the jobs' streams: ") + cudaGetErrorString(e));
 }
 
 rewl_status check_batch(rewl_batch* b) {
@@ -241,8 +246,7 @@ rewl_status check_batch(rewl_batch* b) {
   return REWL_OK;
 }
 
-rewl_status run_intervals(rewl_batch* b, long long n) {
-  if (b->items.empty() || n <= 0) return REWL_OK;
+rewl_status enqueue_intervals(rewl_batch* b, long long n) {
   rewl_status s = order_after_jobs(b);
   if (s != REWL_OK) return s;
   long long left = n;
@@ -263,7 +267,12 @@ rewl_status run_intervals(rewl_batch* b, long long n) {
     left -= step;
     for (int j : b->active_ids) job_add_intervals(b->jobs[j], step);
   }
-  return order_jobs_after(b);
+  return REWL_OK;
+}
+
+rewl_status run_intervals(rewl_batch* b, long long n) {
+  if (b->items.empty() || n <= 0) return REWL_OK;
+  return order_jobs_after(b, enqueue_intervals(b, n));
 }
 
 }  // namespace
@@ -381,18 +390,12 @@ extern "C" rewl_status rewl_batch_set_tuning(rewl_batch* b, const rewl_batch_tun
   return s;
 }
 
-extern "C" rewl_status rewl_batch_autotune(rewl_batch* b, int64_t trial_moves, rewl_batch_tuning* chosen,
-                                           double* ms_out) {
-  NvtxRange nvtx_("rewl_batch_autotune");
-  rewl_status s = check_batch(b);
-  if (s != REWL_OK) return s;
-  if (trial_moves < 1) return bfail(b, REWL_EINVAL, "trial_moves must be > 0");
-  if (b->items.empty()) return bfail(b, REWL_ESTATE, "no active jobs");
+static rewl_status autotune(rewl_batch* b, long long trial_moves, rewl_batch_tuning* chosen, double* ms_out) {
   std::vector<int> thresholds = {0};
   for (int j : b->active_ids) thresholds.push_back(b->view[j].N);
   std::sort(thresholds.begin(), thresholds.end());
   thresholds.erase(std::unique(thresholds.begin(), thresholds.end()), thresholds.end());
-  s = order_after_jobs(b);
+  rewl_status s = order_after_jobs(b);
   if (s != REWL_OK) return s;
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   BCUDA(b, cudaEventCreate(&e0));
@@ -444,8 +447,6 @@ extern "C" rewl_status rewl_batch_autotune(rewl_batch* b, int64_t trial_moves, r
   cudaEventDestroy(e1);
   s = apply_tuning(b, best_w, best_n, best_c);
   if (s != REWL_OK) return s;
-  s = order_jobs_after(b);
-  if (s != REWL_OK) return s;
   if (chosen) {
     chosen->workers_per_block = best_w;
     chosen->smem_lattice_max_n = best_n;
@@ -453,6 +454,16 @@ extern "C" rewl_status rewl_batch_autotune(rewl_batch* b, int64_t trial_moves, r
   }
   if (ms_out) *ms_out = best;
   return REWL_OK;
+}
+
+extern "C" rewl_status rewl_batch_autotune(rewl_batch* b, int64_t trial_moves, rewl_batch_tuning* chosen,
+                                           double* ms_out) {
+  NvtxRange nvtx_("rewl_batch_autotune");
+  const rewl_status s = check_batch(b);
+  if (s != REWL_OK) return s;
+  if (trial_moves < 1) return bfail(b, REWL_EINVAL, "trial_moves must be > 0");
+  if (b->items.empty()) return bfail(b, REWL_ESTATE, "no active jobs");
+  return order_jobs_after(b, autotune(b, trial_moves, chosen, ms_out));
 }
 
 extern "C" rewl_status rewl_batch_run_intervals(rewl_batch* b, int n_intervals) {
@@ -463,12 +474,8 @@ extern "C" rewl_status rewl_batch_run_intervals(rewl_batch* b, int n_intervals) 
   return run_intervals(b, n_intervals);
 }
 
-extern "C" rewl_status rewl_batch_run_to_convergence(rewl_batch* b, int64_t max_intervals, int check_every,
-                                                     int* n_done) {
-  NvtxRange nvtx_("rewl_batch_run_to_convergence");
-  rewl_status s = check_batch(b);
-  if (s != REWL_OK) return s;
-  if (max_intervals < 1 || check_every < 1) return bfail(b, REWL_EINVAL, "max_intervals and check_every must be >= 1");
+static rewl_status run_to_convergence(rewl_batch* b, long long max_intervals, int check_every, int* n_done) {
+  rewl_status s = REWL_OK;
   const int n = (int)b->jobs.size();
   long long done_intervals = 0;
   std::vector<int> cnt;
@@ -507,7 +514,16 @@ extern "C" rewl_status rewl_batch_run_to_convergence(rewl_batch* b, int64_t max_
     done_intervals += k;
   }
   if (n_done) *n_done = count_done();
-  return order_jobs_after(b);
+  return REWL_OK;
+}
+
+extern "C" rewl_status rewl_batch_run_to_convergence(rewl_batch* b, int64_t max_intervals, int check_every,
+                                                     int* n_done) {
+  NvtxRange nvtx_("rewl_batch_run_to_convergence");
+  const rewl_status s = check_batch(b);
+  if (s != REWL_OK) return s;
+  if (max_intervals < 1 || check_every < 1) return bfail(b, REWL_EINVAL, "max_intervals and check_every must be >= 1");
+  return order_jobs_after(b, run_to_convergence(b, max_intervals, check_every, n_done));
 }
 
 extern "C" rewl_status rewl_batch_get_info(const rewl_batch* b, rewl_batch_info* out) {

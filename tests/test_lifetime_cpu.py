@@ -1,0 +1,40 @@
+"""What the library's host code does with device memory and streams where a call fails or a run is closed early,
+on a CUDA runtime without a GPU that keeps account of it (tests/cuda/fake_runtime.cpp)."""
+import pytest
+
+import fake_runtime
+
+JOBS = """
+def job(seed, **kw):
+    return rw.REWL(kind=rw.BCC, L=8, J=(1.0, 0.5), n_bins=200, n_windows=4, walkers_per_window=2, seed=seed,
+                   group_size=1, exchange_interval=100, stream=0, **kw)
+
+def refused(f, *a):
+    try:
+        f(*a)
+    except rw.RewlError as e:
+        return e.status
+    raise AssertionError("the call went through")
+"""
+
+
+@pytest.mark.parametrize("call,skip,run", [
+    ("cudaGraphInstantiate", 1, "b.run_intervals, 9"),          # the graph of eight intervals runs, that of one fails
+    ("cudaGraphLaunch", 1, "b.run_intervals, 9"),
+    ("cudaStreamBeginCapture", 1, "b.run_intervals, 9"),
+    ("cudaEventSynchronize", 1, "b.autotune, 100"),
+    ("cudaMemcpyAsync", 0, "b.run_to_convergence, 8, 8"),
+])
+def test_a_batch_call_that_fails_leaves_its_jobs_ordered_after_it(call, skip, run):
+    fake_runtime.run(JOBS + f"""
+jobs = [job(1), job(2)]
+b = rw.Batch(jobs, stream=0)
+lib.fake_fail(b"{call}", {skip}, 719)
+assert refused({run}) == rw.ECUDA and lib.fake_failed()
+lib.cudaStreamSynchronize(None)        # the jobs' stream
+assert lib.fake_unfinished() == 0
+for j in jobs:
+    j.close()
+b.close()
+assert lib.fake_bad_frees() == 0
+""")
