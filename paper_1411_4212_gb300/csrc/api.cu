@@ -95,6 +95,7 @@ struct rewl_handle {
   double* d_avg = nullptr;
   int32_t* d_bstar = nullptr;
   double* d_merge = nullptr;
+  int device = 0;
   unsigned char* arena = nullptr;   // every array above, one allocation
   size_t walkers_bytes = 0;         // its first part: ln g, H, and from small_begin on the per-slot arrays
   size_t small_begin = 0;
@@ -404,9 +405,14 @@ const char* rewl_last_error(const rewl_handle* h) {
 void rewl_destroy(rewl_handle* h) {
   if (!h) return;
   if (h->arena) {
-    // the handle's stream has waited for every batch that used the arrays
-    cudaStreamSynchronize(h->stream);
+    // whatever still uses the arrays, on whichever stream (a graph that the caller captured, a batch), has to end
+    // before the pool may give them to another run
+    int dev = h->device;
+    cudaGetDevice(&dev);
+    if (dev != h->device) cudaSetDevice(h->device);
+    cudaDeviceSynchronize();
     pool_free(h->arena, nullptr);
+    if (dev != h->device) cudaSetDevice(dev);
   }
   pool_release();
   delete h;
@@ -631,6 +637,7 @@ static rewl_status create_impl(const rewl_lattice* lat, const rewl_couplings* cp
     rewl_destroy(h);
     return REWL_ECUDA;
   }
+  h->device = dev;
   const size_t with_lattice = walker_smem_bytes(h->traj, true, h->N, h->W);
   h->smem_lattice = with_lattice + 1024 <= (size_t)max_smem;
   h->smem_bytes = walker_smem_bytes(h->traj, h->smem_lattice, h->N, h->W);

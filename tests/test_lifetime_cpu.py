@@ -38,3 +38,14 @@ for j in jobs:
 b.close()
 assert lib.fake_bad_frees() == 0
 """)
+
+
+def test_a_run_that_is_closed_waits_for_work_on_other_streams():
+    """Work that the caller has captured or ordered onto a stream of its own may still use the run's arrays."""
+    fake_runtime.run(JOBS + """
+g = job(1)
+other = lib.fake_stream(1)             # does not wait for the legacy stream, nor that one for it
+lib.fake_work(other)
+g.close()
+assert lib.fake_bad_frees() == 0
+""")
