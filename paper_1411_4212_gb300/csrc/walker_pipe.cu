@@ -39,12 +39,14 @@ __device__ __forceinline__ void named_arrive(int id) {
 struct alignas(16) MoveBatch {
   int4 head[32];         // energy increment (2^-24 bins) | ln u (2^-20 units) | moves of batch b-1 touching
                          // this one | earlier moves of this batch touching it (both as they are counted)
-  int4 place[32];        // site | octahedral code (u, v) of the proposed spin, what the lattice stores
+  int4 place[32];        // site | octahedral code (u, v) of the proposed spin, what the lattice stores | half-unit
+                         // coordinates X | Y << 10 | Z << 20 (here, where the resolver writes nothing, because the
+                         // producer reads them of the batch that is being resolved)
   float4 n[32];          // proposed spin | earlier moves of this batch on this site
   float4 h[32];          // local field (snapshot) | moves of batch b-1 on this site (bits reversed: move j
                          // is bit 31 - j, so that count-leading-zeros walks them in order)
   float4 ds[32];         // new - old spin: the move's change to the lattice if accepted (kept current by
-                         // the resolver) | half-unit coordinates X | Y << 10 | Z << 20
+                         // the resolver)
   int4 cur[32];          // earlier moves of this batch on a neighbour, by shell
   int4 prev[32];         // moves of batch b-1 on a neighbour, by shell (bits reversed)
   int4 all;              // moves that touch a later one | moves on a later one's site | moves whose
@@ -353,7 +355,8 @@ __device__ __forceinline__ void pipe_walk_slot(const WalkerArgs& a, const int sl
         const float dx = __fsub_rn(nx, ox), dy = __fsub_rn(ny, oy), dz = __fsub_rn(nz, oz);
         const float dE = -fmaf(dz, hz, fmaf(dy, hy, dx * hx));
         const int dq = dq24_of(dE, a.win);
-        m.ds[lane] = make_float4(dx, dy, dz, __int_as_float(X | (Y << 10) | (Z << 20)));
+        m.ds[lane] = make_float4(dx, dy, dz, 0.0f);
+        m.place[lane] = make_int4(site, __float_as_int(code.x), __float_as_int(code.y), X | (Y << 10) | (Z << 20));
         if (aliased) {
           // An owner table smaller than the lattice is hashed: a bit may name a move whose site is neither
           // this move's site nor one of its neighbours, or name a shell that it does not sit on.  Sort the
@@ -364,7 +367,7 @@ __device__ __forceinline__ void pipe_walk_slot(const WalkerArgs& a, const int sl
             same = sh[0] = sh[1] = sh[2] = sh[3] = 0u;
             for (; bits; bits &= bits - 1u) {
               const int j = __ffs(bits) - 1;
-              const uint32_t q = __float_as_uint(other.ds[j].w), bit = 1u << j;
+              const uint32_t q = (uint32_t)other.place[j].w, bit = 1u << j;
               // every offset component of a neighbour is below L half-units, so the wrapped displacement
               // is the offset; squared distances 3, 4, 8, 11 are the shells 1..4
               int ex = abs((int)(q & 1023u) - X), ey = abs((int)((q >> 10) & 1023u) - Y), ez = abs((int)(q >> 20) - Z);
@@ -388,7 +391,6 @@ __device__ __forceinline__ void pipe_walk_slot(const WalkerArgs& a, const int sl
           }
         }
         m.head[lane] = make_int4(dq, lu, (int)cprev, (int)ccur);
-        m.place[lane] = make_int4(site, __float_as_int(code.x), __float_as_int(code.y), 0);
         m.n[lane] = make_float4(nx, ny, nz, __uint_as_float(scur));
         m.h[lane] = make_float4(hx, hy, hz, __uint_as_float(__brev(sprev)));
         m.cur[lane] = make_int4((int)tcur[0], (int)tcur[1], (int)tcur[2], (int)tcur[3]);
@@ -757,6 +759,8 @@ __device__ __forceinline__ void pipe_walk_slot(const WalkerArgs& a, const int sl
       // d = ln g(now) - ln g(target) in 2^-40 units this is d >= 0 or ln u < floor(d / 2^20).  With
       // ln g(now) = A + lane ln f: ln g(target) <= A + Q.
       const long long Q = lane_lnf - (hd.y < 0 ? (long long)(hd.y + 1) * 1048576LL : 0LL);
+      // (it reads what an earlier push of the batch may have written in another lane: the warp is ordered before it,
+      // with nothing to wait for there; after the store the same barrier cost 2 % of a batch, 7 % in the dense form)
       auto push = [&](const int e) {
         const uint32_t bit = 1u << e;
         const float4 de = C.ds[e];
@@ -813,6 +817,7 @@ __device__ __forceinline__ void pipe_walk_slot(const WalkerArgs& a, const int sl
           // stays passes the test too
           const bool ok = live && (unsigned)rel < (unsigned)W && lt <= A + Q;
           const uint32_t m = __reduce_min_sync(kFullMask, ok ? key : kNoKey);
+          __syncwarp();                    // for push, below
           const int e = (int)(m >> 27);
           const long long A2 = shfl_ll(rel == r ? A : lt - lane_lnf, e);   // ln g after the move, less e ln f
           int pe = frac + ((int)(m << 5) >> 5);
@@ -873,6 +878,7 @@ __device__ __forceinline__ void pipe_walk_slot(const WalkerArgs& a, const int sl
             rn = r0;
             key = lane > e ? key : kNoKey;
             if ((touched >> e) & 1u) {
+              __syncwarp();
               push(e);
               key = key == kNoKey ? kNoKey : make_key();
             }
@@ -927,7 +933,10 @@ __device__ __forceinline__ void pipe_walk_slot(const WalkerArgs& a, const int sl
             }
             acc_cur |= 1u << e;
             frac = pe & (kBin - 1);
-            if ((touched >> e) & 1u) push(e);
+            if ((touched >> e) & 1u) {
+              __syncwarp();
+              push(e);
+            }
             arm();
           } else {
             live = live && lane > e;
