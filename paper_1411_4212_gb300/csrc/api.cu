@@ -113,8 +113,10 @@ struct rewl_handle {
 // device's default pool (whose settings belong to the host program).  A fresh cudaMalloc, or an allocation
 // from a pool that has given everything back, costs 50 to 300 us on GB300; a run's handle needs some 25
 // arrays, and thermodynamics, joining and the network's calls need scratch every time.  The pool keeps at
-// most 64 MiB that is not in use, and 4 MiB once the last handle and model are gone.  It is safe with several
-// threads and streams: the driver orders a block's next use after its last.
+// most 64 MiB that is not in use.  When the last handle or model goes it is cut to 4 MiB (the driver reserves
+// pieces of 32 MiB: to one of them), or to what calls in other threads have at that moment; calls without a
+// handle may fill it to 64 MiB again.  It is safe with several threads and streams: the driver orders a block's
+// next use after its last.
 namespace {
 
 constexpr int kMaxDevices = 128;
@@ -160,7 +162,10 @@ cudaError_t rewl::pool_alloc(void** p, size_t bytes, cudaStream_t stream) {
 }
 
 void rewl::pool_free(void* p, cudaStream_t stream) {
-  if (p) cudaFreeAsync(p, stream);
+  if (!p || cudaFreeAsync(p, stream) == cudaSuccess) return;
+  cudaGetLastError();
+  cudaStreamSynchronize(stream);
+  cudaFree(p);
 }
 
 void rewl::pool_retain() {
@@ -411,7 +416,7 @@ void rewl_destroy(rewl_handle* h) {
     cudaGetDevice(&dev);
     if (dev != h->device) cudaSetDevice(h->device);
     cudaDeviceSynchronize();
-    pool_free(h->arena, nullptr);
+    cudaFree(h->arena);              // at once, so that pool_release can trim it
     if (dev != h->device) cudaSetDevice(dev);
   }
   pool_release();

@@ -49,3 +49,41 @@ lib.fake_work(other)
 g.close()
 assert lib.fake_bad_frees() == 0
 """)
+
+
+LARGE = """
+def large(seed):
+    return rw.REWL(kind=rw.BCC, L=16, J=(1.0, 0.5), n_bins=400, n_windows=8, walkers_per_window=100, group_size=1,
+                   stream=0, seed=seed)
+"""
+
+
+def test_what_the_pool_keeps_once_nobody_uses_it():
+    """Runs of 52 MB of lattices: while another one lives the pool keeps them (it keeps up to 64 MiB), once the last
+    one is gone 4 MiB are left, whatever its size.  A model's scratch counts too."""
+    fake_runtime.run(JOBS + LARGE + """
+a, b = large(1), job(2)
+a.close()
+assert lib.fake_pool_reserved() > 50 << 20
+a = large(3)
+b.close()
+assert lib.fake_pool_reserved() > 50 << 20
+a.close()
+assert lib.fake_pool_reserved() <= 4 << 20
+m = rw.Mlp(np.zeros(6, np.float32), np.ones(6, np.float32), stream=0)
+m.forward(np.zeros((1 << 20, 6), np.float32))
+assert lib.fake_pool_reserved() > 25 << 20
+m.close()
+assert lib.fake_pool_reserved() <= 4 << 20
+""")
+
+
+def test_scratch_that_a_stream_refuses_to_free_is_not_lost():
+    fake_runtime.run("""
+m = rw.Mlp(np.zeros(6, np.float32), np.ones(6, np.float32), stream=0)
+lib.fake_fail(b"cudaFreeAsync", 0, 719)
+m.forward(np.zeros((1 << 20, 6), np.float32))
+assert lib.fake_failed()
+m.close()
+assert lib.fake_pool_reserved() <= 4 << 20 and lib.fake_bad_frees() == 0
+""")
