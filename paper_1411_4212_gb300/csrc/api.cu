@@ -157,8 +157,10 @@ cudaError_t device_pool(cudaMemPool_t* pool) {
 cudaError_t rewl::pool_alloc(void** p, size_t bytes, cudaStream_t stream) {
   *p = nullptr;
   cudaMemPool_t pool = nullptr;
-  const cudaError_t e = device_pool(&pool);
-  return e == cudaSuccess ? cudaMallocFromPoolAsync(p, std::max<size_t>(bytes, 1), pool, stream) : e;
+  cudaError_t e = device_pool(&pool);
+  if (e == cudaSuccess) e = cudaMallocFromPoolAsync(p, std::max<size_t>(bytes, 1), pool, stream);
+  if (e == cudaErrorMemoryAllocation) cudaGetLastError();   // reported here, not by the next launch's check
+  return e;
 }
 
 void rewl::pool_free(void* p, cudaStream_t stream) {

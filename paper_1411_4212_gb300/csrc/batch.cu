@@ -71,7 +71,10 @@ template <class T>
 rewl_status balloc(rewl_batch* b, T** p, size_t count) {
   void* q = nullptr;
   cudaError_t e = cudaMalloc(&q, std::max<size_t>(count, 1) * sizeof(T));
-  if (e != cudaSuccess) return bfail(b, REWL_ENOMEM, std::string("cudaMalloc: ") + cudaGetErrorString(e));
+  if (e != cudaSuccess) {
+    cudaGetLastError();          // (the jobs stay usable: their next launch's check must not find this)
+    return bfail(b, REWL_ENOMEM, std::string("cudaMalloc: ") + cudaGetErrorString(e));
+  }
   b->allocations.push_back(q);
   *p = static_cast<T*>(q);
   return REWL_OK;

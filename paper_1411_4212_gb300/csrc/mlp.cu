@@ -788,7 +788,10 @@ template <class T>
 rewl_status malloc_dev(rewl_mlp* m, T** p, size_t count) {
   void* q = nullptr;
   const cudaError_t e = cudaMalloc(&q, std::max<size_t>(count, 1) * sizeof(T));
-  if (e != cudaSuccess) return mfail(m, REWL_ENOMEM, std::string("cudaMalloc: ") + cudaGetErrorString(e));
+  if (e != cudaSuccess) {
+    cudaGetLastError();          // (the model stays usable: the next launch's check must not find this)
+    return mfail(m, REWL_ENOMEM, std::string("cudaMalloc: ") + cudaGetErrorString(e));
+  }
   m->allocations.push_back(q);
   *p = static_cast<T*>(q);
   return REWL_OK;
@@ -1028,16 +1031,17 @@ extern "C" rewl_status rewl_mlp_train(rewl_mlp* m, const float* x, const float* 
   if (loss_history) MCUDA(m, c.sc.get(&d_loss, (size_t)steps));
   const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
   for (int it = 0; it < steps; ++it) {
-    m->adam_t += 1;
+    const long long step = m->adam_t + 1;
     AdamArgs a{};
     a.lr = lr;
     a.b1 = b1;
     a.b2 = b2;
     a.eps = eps;
-    a.c1 = 1.0f - std::pow(b1, (float)m->adam_t);
-    a.c2 = 1.0f - std::pow(b2, (float)m->adam_t);
+    a.c1 = 1.0f - std::pow(b1, (float)step);
+    a.c2 = 1.0f - std::pow(b2, (float)step);
     s = loss_and_grad(m, c.x, c.t, c.seg, n_runs, n, c.y, c.dy, c.loss, d_loss ? d_loss + it : nullptr, &a);
     if (s != REWL_OK) return s;
+    m->adam_t = step;
   }
   if (loss_history) {
     std::vector<double> loss((size_t)steps);

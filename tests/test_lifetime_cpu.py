@@ -87,3 +87,35 @@ assert lib.fake_failed()
 m.close()
 assert lib.fake_pool_reserved() <= 4 << 20 and lib.fake_bad_frees() == 0
 """)
+
+
+def test_training_that_runs_out_of_memory_can_be_tried_again():
+    """The first gradient allocates; where that fails the model stays usable, the retry's first step is Adam's first
+    one, and no error is left for the next call to find."""
+    fake_runtime.run(JOBS + """
+m = rw.Mlp(np.zeros(6, np.float32), np.ones(6, np.float32), stream=0)
+args = (np.zeros((10, 6), np.float32), np.zeros(10, np.float32), np.array([0, 10], np.int32))
+lib.fake_fail(b"cudaMalloc", 0, 2)
+assert refused(m.train, *args, 3, 1e-3) == rw.ENOMEM and lib.fake_failed()
+lib.fake_watch(b"mlp_reduce_kernel", 11, 24)
+m.train(*args, 2, 1e-3)
+adam = (ctypes.c_float * 6)()
+for i in range(2):
+    assert lib.fake_seen(i, adam) == 2
+    assert abs(adam[4] - (1 - 0.9 ** (i + 1))) < 1e-6, list(adam)
+m.close()
+""")
+
+
+@pytest.mark.parametrize("call", ["cudaMallocFromPoolAsync", "cudaMalloc"])
+def test_creating_something_without_memory_leaves_no_error_behind(call):
+    fake_runtime.run(JOBS + f"""
+make = (lambda: job(1)) if "{call}" == "cudaMallocFromPoolAsync" else (lambda: rw.Batch([g], stream=0))
+g = job(2)
+g.init_walkers()
+lib.fake_fail(b"{call}", 0, 2)
+assert refused(make) == rw.ENOMEM and lib.fake_failed()
+g.run_intervals(1)
+make().close()
+g.close()
+""")
