@@ -764,6 +764,7 @@ struct rewl_mlp {
   float* d_v = nullptr;
   float* d_partial = nullptr;
   float* d_chunk = nullptr;      // activations and dL/dZ of one chunk of samples, allocated by the first gradient
+  long long chunk_rows = 0;      // samples that d_chunk holds
   int grid = 0;                  // CTAs of a pass over the samples (= rows of d_partial)
   long long adam_t = 0;
   std::vector<void*> allocations;
@@ -836,20 +837,35 @@ rewl_status check_segments(const int32_t* seg, int n_segs, long long n) {
   return REWL_OK;
 }
 
+// Room in d_chunk for `rows` samples, of `most` that are ever needed at once.  It grows by half at least, so that
+// larger and larger corpora seldom allocate.
+rewl_status reserve_chunk(rewl_mlp* m, long long rows, long long most) {
+  if (rows <= m->chunk_rows) return REWL_OK;
+  rows = std::min(most, std::max(rows, m->chunk_rows + m->chunk_rows / 2));
+  cudaFree(m->d_chunk);
+  m->d_chunk = nullptr;
+  m->chunk_rows = 0;
+  const cudaError_t e = cudaMalloc(&m->d_chunk, 5 * (size_t)rows * kH * sizeof(float));
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    return mfail(m, REWL_ENOMEM, std::string("cudaMalloc: ") + cudaGetErrorString(e));
+  }
+  m->chunk_rows = rows;
+  return REWL_OK;
+}
+
 // Loss and gradient of the full batch into m->d_grad, the loss (FP32) into *d_loss when given; with adam,
 // one step of the parameters too.  Stream-ordered.
 rewl_status loss_and_grad(rewl_mlp* m, const float* dx, const float* dt, const int* dseg, int n_segs, long long n,
                           float* dy_buf, float* dydy, double* dloss, double* d_loss, const AdamArgs* adam) {
   const long long chunk = 2LL * m->grid * kWarps * kT;   // two rounds of the backward pass: about 100 MB, in the L2
-  if (!m->d_chunk) {
-    const rewl_status s = malloc_dev(m, &m->d_chunk, 5 * (size_t)chunk * kH);
-    if (s != REWL_OK) return s;
-  }
+  const rewl_status s = reserve_chunk(m, std::min(n, chunk), chunk);
+  if (s != REWL_OK) return s;
   mlp_fwd_kernel<<<fwd_grid(m, n), kThreads, sizeof(Weights), m->stream>>>(m->net, dx, n, dy_buf);
   MCUDA(m, cudaGetLastError());
   mlp_loss_kernel<<<n_segs, 256, 0, m->stream>>>(dy_buf, dt, dseg, (double)n, dydy, dloss);
   MCUDA(m, cudaGetLastError());
-  const Chunk c = Chunk::of(m->d_chunk, chunk);
+  const Chunk c = Chunk::of(m->d_chunk, m->chunk_rows);
   for (long long s0 = 0; s0 < n; s0 += chunk) {
     const int n_c = (int)std::min<long long>(chunk, n - s0);
     const int first = s0 == 0 ? 1 : 0;
@@ -1097,6 +1113,7 @@ extern "C" void rewl_mlp_destroy(rewl_mlp* m) {
   if (!m) return;
   if (!m->broken) cudaStreamSynchronize(m->stream);
   for (void* p : m->allocations) cudaFree(p);
+  cudaFree(m->d_chunk);
   pool_release();
   delete m;
 }

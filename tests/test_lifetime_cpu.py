@@ -119,3 +119,19 @@ g.run_intervals(1)
 make().close()
 g.close()
 """)
+
+
+def test_a_model_holds_no_more_scratch_than_its_samples_need():
+    """2.5 KB per sample for the backward pass, at most two rounds of all CTAs (38912 samples); it grows with the
+    largest gradient so far, by half at least, and is freed with the model."""
+    fake_runtime.run(JOBS + """
+m = rw.Mlp(np.zeros(6, np.float32), np.ones(6, np.float32), stream=0)
+base, row, full = lib.fake_plain_bytes(), 5 * 128 * 4, 2 * 152 * 8 * 16
+held = []
+for n in (10, 7, 1000, 1001, 5, full + 1, 3 * full):
+    m.gradient(np.zeros((n, 6), np.float32), np.zeros(n, np.float32), np.array([0, n], np.int32))
+    held.append((lib.fake_plain_bytes() - base) // row)
+assert held == [10, 10, 1000, 1500, 1500, full, full], held
+m.close()
+assert lib.fake_plain_bytes() == 0
+""")
