@@ -7,6 +7,7 @@
 #include <cmath>
 #include <cstring>
 #include <mutex>
+#include <new>
 #include <string>
 #include <vector>
 
@@ -384,10 +385,20 @@ rewl_status check_whole(rewl_handle* h) {
 struct Walkers {
   std::vector<unsigned char> buf;
   const unsigned char* from = nullptr;
-  rewl_status read(rewl_handle* h, bool tables) {
+  // room for the copy, for calls that should fail here and not after their work
+  rewl_status room(rewl_handle* h, bool tables) {
     const size_t begin = tables ? 0 : h->small_begin;
     from = h->arena + begin;
-    buf.resize(h->walkers_bytes - begin);
+    try {
+      buf.resize(h->walkers_bytes - begin);
+    } catch (const std::bad_alloc&) {
+      return fail(h, REWL_ENOMEM, "no host memory to read the walkers back into");
+    }
+    return REWL_OK;
+  }
+  rewl_status read(rewl_handle* h, bool tables) {
+    const rewl_status s = room(h, tables);
+    if (s != REWL_OK) return s;
     CUDA_TRY(h, cudaMemcpyAsync(buf.data(), from, buf.size(), cudaMemcpyDeviceToHost, h->stream));
     CUDA_TRY(h, cudaStreamSynchronize(h->stream));
     return REWL_OK;
@@ -1080,6 +1091,7 @@ rewl_status rewl_run_intervals(rewl_handle* h, int n, rewl_stage_stats* stats) {
   Walkers before, after;
   if (stats) {
     s = before.read(h, false);
+    if (s == REWL_OK) s = after.room(h, false);
     if (s != REWL_OK) return s;
   }
   s = enqueue_intervals(h, n);
@@ -1104,6 +1116,7 @@ rewl_status rewl_run_stage(rewl_handle* h, rewl_stage_stats* stats) {
   const auto t0 = std::chrono::steady_clock::now();
   Walkers before, now;
   s = before.read(h, false);
+  if (s == REWL_OK) s = now.room(h, false);
   if (s != REWL_OK) return s;
   long long moves_per_walker = 0;
   int intervals = 0;
@@ -1149,9 +1162,11 @@ rewl_status rewl_exchange(rewl_handle* h, rewl_stage_stats* stats) {
   ea.ex = h->ex;
   ea.key1 = h->key1;
   ea.traj = h->traj ? 1 : 0;
+  Walkers w;
+  if (stats) s = w.room(h, false);
+  if (s != REWL_OK) return s;
   CUDA_TRY(h, launch_exchange(ea, h->stream));
   if (stats) {
-    Walkers w;
     s = w.read(h, false);
     if (s != REWL_OK) return s;
     fill_stats(h, w, stats, 0, 0, 0, 0.0);
@@ -1240,11 +1255,16 @@ rewl_status rewl_thermo(const double* lng, const double* centres, int B, double 
   for (int i = 0; i < nT; ++i)
     if (!(T[i] > 0)) return fail(nullptr, REWL_EINVAL, "temperatures must be > 0");
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
+  std::vector<double> out;
+  try {
+    out.resize(3 * (size_t)nT);
+  } catch (const std::bad_alloc&) {
+    return fail(nullptr, REWL_ENOMEM, "no host memory for the results of thermo");
+  }
   double* d = nullptr;
   const size_t bytes = sizeof(double) * (2 * (size_t)B + 4 * (size_t)nT);
   cudaError_t e = pool_alloc(reinterpret_cast<void**>(&d), bytes, st);
   if (e != cudaSuccess) return fail(nullptr, REWL_ENOMEM, "thermo scratch allocation failed");
-  std::vector<double> out(3 * (size_t)nT);
   double *dl = d, *dE = d + B, *dT = d + 2 * B, *dU = dT + nT, *dC = dU + nT, *dZ = dC + nT;
   e = cudaMemcpyAsync(dl, lng, sizeof(double) * B, cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess) e = cudaMemcpyAsync(dE, centres, sizeof(double) * B, cudaMemcpyHostToDevice, st);

@@ -42,6 +42,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <new>
 #include <random>
 #include <string>
 #include <vector>
@@ -1043,6 +1044,12 @@ extern "C" rewl_status rewl_mlp_train(rewl_mlp* m, const float* x, const float* 
   Corpus c(m);
   s = upload_corpus(m, c, x, target, run_offsets, n_runs);
   if (s != REWL_OK) return s;
+  std::vector<double> loss;
+  try {
+    if (loss_history) loss.resize((size_t)steps);
+  } catch (const std::bad_alloc&) {
+    return mfail(m, REWL_ENOMEM, "no host memory for the loss history");
+  }
   double* d_loss = nullptr;      // loss before each step
   if (loss_history) MCUDA(m, c.sc.get(&d_loss, (size_t)steps));
   const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
@@ -1060,7 +1067,6 @@ extern "C" rewl_status rewl_mlp_train(rewl_mlp* m, const float* x, const float* 
     m->adam_t = step;
   }
   if (loss_history) {
-    std::vector<double> loss((size_t)steps);
     MCUDA(m, cudaMemcpyAsync(loss.data(), d_loss, sizeof(double) * (size_t)steps, cudaMemcpyDeviceToHost, m->stream));
     MCUDA(m, cudaStreamSynchronize(m->stream));
     for (int it = 0; it < steps; ++it) loss_history[it] = (float)loss[it];

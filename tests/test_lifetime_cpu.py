@@ -135,3 +135,27 @@ assert held == [10, 10, 1000, 1500, 1500, full, full], held
 m.close()
 assert lib.fake_plain_bytes() == 0
 """)
+
+
+@pytest.mark.parametrize("call", [
+    "rw.thermo(np.zeros(100), np.linspace(-1, 0, 100), 10, np.linspace(1, 2, 100000), stream=0)",
+    "traj.walkers()",
+    "traj.run_intervals(1)",
+    "traj.exchange()",
+    "m.train(np.zeros((10, 6), np.float32), np.zeros(10, np.float32), np.array([0, 10], np.int32), 200000, 1e-3)",
+])
+def test_host_memory_that_is_refused_is_a_status(call):
+    """Read-backs go through host memory of the library's: without it a call returns REWL_ENOMEM (an exception would
+    not get past the C interface) and leaves the run or the model as it was."""
+    fake_runtime.run(JOBS + f"""
+traj = rw.REWL(kind=rw.BCC, L=4, J=(1.0,), n_bins=80, n_windows=4, walkers_per_window=4000, mode=rw.TRAJECTORY,
+               stream=0, seed=1)
+traj.run_intervals(1, stats=False)
+m = rw.Mlp(np.zeros(6, np.float32), np.ones(6, np.float32), stream=0)
+lib.fake_refuse_from(1 << 20)
+assert refused(lambda: {call}) == rw.ENOMEM
+lib.fake_refuse_from(1 << 62)
+{call}
+traj.close()
+m.close()
+""")
