@@ -148,7 +148,7 @@ def test_host_memory_that_is_refused_is_a_status(call):
     """Read-backs go through host memory of the library's: without it a call returns REWL_ENOMEM (an exception would
     not get past the C interface) and leaves the run or the model as it was."""
     fake_runtime.run(JOBS + f"""
-traj = rw.REWL(kind=rw.BCC, L=4, J=(1.0,), n_bins=80, n_windows=4, walkers_per_window=4000, mode=rw.TRAJECTORY,
+traj = rw.REWL(kind=rw.BCC, L=4, J=(1.0,), n_bins=80, n_windows=4, walkers_per_window=6000, mode=rw.TRAJECTORY,
                stream=0, seed=1)
 traj.run_intervals(1, stats=False)
 m = rw.Mlp(np.zeros(6, np.float32), np.ones(6, np.float32), stream=0)
