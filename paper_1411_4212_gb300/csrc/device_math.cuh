@@ -47,4 +47,13 @@ __device__ __forceinline__ unsigned long long pow2_entry(int j) {
   return v;
 }
 
+// 1 / d for 1 <= d <= 2^126, by Newton's iteration r' = r + r (1 - d r) from the hardware's estimate (relative
+// error e = 2^-23): one step leaves e^2 and its own rounding, so at most one unit in the last place.  Where 1 / d
+// is below the smallest normal number it is 0.
+__device__ __forceinline__ float reciprocal(float d) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(d));
+  return fmaf(fmaf(-d, r, 1.0f), r, r);
+}
+
 }  // namespace rewl

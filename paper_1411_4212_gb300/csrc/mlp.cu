@@ -48,6 +48,7 @@
 #include <vector>
 
 #include "../../include/rewl.h"
+#include "device_math.cuh"
 #include "jobs.h"
 #include "walker.h"
 
@@ -75,18 +76,6 @@ struct Net {
   const __nv_bfloat16* p;    // BF16 parameters
   float shift[kIn], scale[kIn];
 };
-
-__device__ __forceinline__ float rcp_estimate(float x) {
-  float r;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-  return r;
-}
-
-// 1 / d, d >= 1: the hardware's estimate with one Newton step, within one unit in the last place.
-__device__ __forceinline__ float reciprocal(float d) {
-  const float r = rcp_estimate(d);
-  return fmaf(fmaf(-d, r, 1.0f), r, r);
-}
 
 // 1 / (1 + e^-z).  Below z = -88, where e^-z would overflow, the value there (6e-39 or 0) stands for it.
 __device__ __forceinline__ float sigmoid(float z) { return reciprocal(1.0f + expf(-fmaxf(z, -88.0f))); }

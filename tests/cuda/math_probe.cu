@@ -8,6 +8,10 @@ __global__ void exp_kernel(const double* x, double* y, int n) {
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) y[i] = rewl::exp_fixed(x[i], pow2);
 }
 
+__global__ void reciprocal_kernel(const float* x, float* y, int n) {
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) y[i] = rewl::reciprocal(x[i]);
+}
+
 template <class T, class F>
 static int apply(const T* x, T* y, int n, F launch) {
   T *dx = nullptr, *dy = nullptr;
@@ -26,4 +30,7 @@ static int apply(const T* x, T* y, int n, F launch) {
 
 extern "C" int probe_exp(const double* x, double* y, int n) {
   return apply(x, y, n, [n](const double* a, double* b) { exp_kernel<<<256, 256>>>(a, b, n); });
+}
+extern "C" int probe_reciprocal(const float* x, float* y, int n) {
+  return apply(x, y, n, [n](const float* a, float* b) { reciprocal_kernel<<<256, 256>>>(a, b, n); });
 }

@@ -37,3 +37,21 @@ def test_exponential_of_the_thermodynamics():
     far = _apply("probe_exp", np.array([-708.0, np.nextafter(-708.0, -1000), -1e4, -1e308, -np.inf]))
     assert np.array_equal(far, np.zeros(5))
     assert np.isnan(_apply("probe_exp", np.array([np.nan]))).all()
+
+
+def test_reciprocal_of_the_network():
+    """1 / d for d in [1, 2^126], all exponents and the values that sigmoids see, within one unit in the last place; 0
+    beyond, where 1 / d is no normal number any more."""
+    rng = np.random.default_rng(2)
+    powers = 2.0 ** np.arange(0, 127)
+    d = np.concatenate([powers, np.exp2(rng.uniform(0, 126, 500000)), 1 + np.exp(rng.uniform(-20, 87, 500000)),
+                        1 + np.arange(1 << 16) * 2.0 ** -23]).astype(np.float32)
+    d = np.unique(np.concatenate([d, np.nextafter(d, np.float32(0))]))
+    d = d[(d >= 1) & (d <= np.float32(2.0 ** 126))]
+    r = _apply("probe_reciprocal", d).astype(np.float64)
+    exact = 1.0 / d.astype(np.float64)
+    unit = np.spacing(np.nextafter(exact.astype(np.float32), np.float32(0))).astype(np.float64)
+    err = np.abs(r - exact) / unit
+    assert err.max() <= 1.0, (d[err.argmax()], err.max())
+    beyond = np.array([np.nextafter(np.float32(2.0 ** 126), np.float32(3e38)), 1.5e38, 1 + np.exp(88.0)], dtype=np.float32)
+    assert np.array_equal(_apply("probe_reciprocal", beyond), np.zeros(3, dtype=np.float32))
