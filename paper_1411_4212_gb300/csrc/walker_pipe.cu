@@ -747,10 +747,16 @@ __device__ __forceinline__ void pipe_walk_slot(const WalkerArgs& a, const int sl
       // Measured (cycles per batch): blocks 350 + 95 per accepted move + 350 per bin change (and per move
       // of a bin or more, if undecided by the pass bits), scan 450 + 100 per rejected exit + 300 per other
       // event, sequential 300 + 160 per accepted move (250 where every accepted move is pushed).  So two
-      // bin changes, or two moves that may reach beyond the next bin, make the sequential path the
-      // cheaper one; between the other two the counts of exits and of accepted moves decide.
-      path = forced >= 0 ? forced
-                         : (n_chg >= 2 || all.z >= 2 ? kSequential : (n_exit + 2 < n_in ? kScan : kBlocks));
+      // bin changes, or two moves that may reach beyond the next bin, make the sequential path cheaper than
+      // blocks; than scan only where few moves are accepted between such events (at the beginning of a run nearly
+      // all are: the first 3 x 1000 moves of bcc L = 16, 1 shell, 500 bins took 125 us each without this comparison,
+      // 81 with it, those of L = 24, 2 shells, 2000 bins 125 and 89).  It asks for a third more than break-even:
+      // counts of the batch before say only so much about this one.  Between scan and blocks the counts of exits and
+      // of accepted moves decide.
+      path = n_chg >= 2 || all.z >= 2 ? kSequential : (n_exit + 2 < n_in ? kScan : kBlocks);
+      const int events = n_chg + __popc(touched) + all.z;
+      if (path == kSequential && 150 + 100 * (n_exit - n_chg) + 300 * events < 110 * n_in) path = kScan;
+      if (forced >= 0) path = forced;
       uint32_t same = 0u;                  // accepted moves of this batch on this lane's site
       uint32_t acc_cur = 0u;
       int rb = r;                          // bin before this lane's move
