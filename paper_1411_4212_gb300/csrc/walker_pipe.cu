@@ -363,28 +363,35 @@ __device__ __forceinline__ void pipe_walk_slot(const WalkerArgs& a, const int sl
           // bits by the distance of the sites.  With the lattice in global memory only real conflicts
           // count.  (At bcc L = 32 with 2048 entries, 92 % of the flagged moves were aliases.)
           __syncwarp();
-          auto sort_bits = [&](const MoveBatch& other, uint32_t bits, uint32_t& same, uint32_t (&sh)[4]) {
-            same = sh[0] = sh[1] = sh[2] = sh[3] = 0u;
-            for (; bits; bits &= bits - 1u) {
-              const int j = __ffs(bits) - 1;
-              const uint32_t q = (uint32_t)other.place[j].w, bit = 1u << j;
-              // every offset component of a neighbour is below L half-units, so the wrapped displacement
-              // is the offset; squared distances 3, 4, 8, 11 are the shells 1..4
-              int ex = abs((int)(q & 1023u) - X), ey = abs((int)((q >> 10) & 1023u) - Y), ez = abs((int)(q >> 20) - Z);
-              ex = min(ex, 2 * L - ex);
-              ey = min(ey, 2 * L - ey);
-              ez = min(ez, 2 * L - ez);
-              const int r2 = ex * ex + ey * ey + ez * ez;
-              // (a shell without coupling changes nothing either)
-              same |= r2 == 0 ? bit : 0u;
-              sh[0] |= r2 == 3 && Jsh[0] != Real(0) ? bit : 0u;
-              sh[1] |= NSH > 1 && r2 == 4 && Jsh[1] != Real(0) ? bit : 0u;
-              sh[2] |= NSH > 2 && r2 == 8 && Jsh[2] != Real(0) ? bit : 0u;
-              sh[3] |= NSH > 3 && r2 == 11 && Jsh[3] != Real(0) ? bit : 0u;
-            }
+          // Both masks in one loop: their moves' words are in flight together (64 runs in a batch 30.6 -> 30.1 ms).
+          uint32_t bc = ccur, bp = cprev;
+          const MoveBatch& before = mb[cur ^ 1];
+          scur = sprev = 0u;
+#pragma unroll
+          for (int s2 = 0; s2 < 4; ++s2) tcur[s2] = tprev[s2] = 0u;
+          auto sort_bit = [&](const uint32_t q, const uint32_t bit, uint32_t& same, uint32_t (&sh)[4]) {
+            // every offset component of a neighbour is below L half-units, so the wrapped displacement
+            // is the offset; squared distances 3, 4, 8, 11 are the shells 1..4
+            int ex = abs((int)(q & 1023u) - X), ey = abs((int)((q >> 10) & 1023u) - Y), ez = abs((int)(q >> 20) - Z);
+            ex = min(ex, 2 * L - ex);
+            ey = min(ey, 2 * L - ey);
+            ez = min(ez, 2 * L - ez);
+            const int r2 = ex * ex + ey * ey + ez * ez;
+            // (a shell without coupling changes nothing either)
+            same |= r2 == 0 ? bit : 0u;
+            sh[0] |= r2 == 3 && Jsh[0] != Real(0) ? bit : 0u;
+            sh[1] |= NSH > 1 && r2 == 4 && Jsh[1] != Real(0) ? bit : 0u;
+            sh[2] |= NSH > 2 && r2 == 8 && Jsh[2] != Real(0) ? bit : 0u;
+            sh[3] |= NSH > 3 && r2 == 11 && Jsh[3] != Real(0) ? bit : 0u;
           };
-          sort_bits(m, ccur, scur, tcur);
-          sort_bits(mb[cur ^ 1], cprev, sprev, tprev);
+          while (bc | bp) {
+            const uint32_t bit_c = bc & (0u - bc), bit_p = bp & (0u - bp);   // 0: none left
+            const uint32_t qc = (uint32_t)m.place[(__ffs(bc) - 1) & 31].w, qp = (uint32_t)before.place[(__ffs(bp) - 1) & 31].w;
+            sort_bit(qc, bit_c, scur, tcur);
+            sort_bit(qp, bit_p, sprev, tprev);
+            bc ^= bit_c;
+            bp ^= bit_p;
+          }
           if constexpr (!kSmem) {
             ccur = scur | tcur[0] | tcur[1] | tcur[2] | tcur[3];
             cprev = sprev | tprev[0] | tprev[1] | tprev[2] | tprev[3];
