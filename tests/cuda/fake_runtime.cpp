@@ -145,6 +145,7 @@ int fake_failed() { return st().fail_call.empty(); }
 long fake_bad_frees() { return st().bad_frees; }
 long fake_unfinished() { return (long)st().unfinished.size(); }
 size_t fake_pool_reserved() { return st().reserved; }
+size_t fake_pool_used() { return st().used; }
 size_t fake_plain_bytes() { return st().plain; }
 long fake_launches() { return st().launches; }
 void fake_refuse_from(size_t bytes) { refuse_from = bytes; }

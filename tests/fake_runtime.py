@@ -14,7 +14,7 @@ sys.modules["torch"] = None
 import numpy as np
 import paper_1411_4212_gb300 as rw
 lib = rw.load_library({out!r})
-lib.fake_pool_reserved.restype = lib.fake_plain_bytes.restype = lib.fake_stream.restype = ctypes.c_size_t
+lib.fake_pool_reserved.restype = lib.fake_pool_used.restype = lib.fake_plain_bytes.restype = lib.fake_stream.restype = ctypes.c_size_t
 lib.fake_refuse_from.argtypes = [ctypes.c_size_t]
 lib.fake_work.argtypes = [ctypes.c_size_t]
 """

@@ -95,7 +95,7 @@ def test_training_that_runs_out_of_memory_can_be_tried_again():
     fake_runtime.run(JOBS + """
 m = rw.Mlp(np.zeros(6, np.float32), np.ones(6, np.float32), stream=0)
 args = (np.zeros((10, 6), np.float32), np.zeros(10, np.float32), np.array([0, 10], np.int32))
-lib.fake_fail(b"cudaMalloc", 0, 2)
+lib.fake_fail(b"cudaMallocFromPoolAsync", 7, 2)     # after the corpus, six arrays, and the loss history
 assert refused(m.train, *args, 3, 1e-3) == rw.ENOMEM and lib.fake_failed()
 lib.fake_watch(b"mlp_reduce_kernel", 11, 24)
 m.train(*args, 2, 1e-3)
@@ -126,14 +126,14 @@ def test_a_model_holds_no_more_scratch_than_its_samples_need():
     largest gradient so far, by half at least, and is freed with the model."""
     fake_runtime.run(JOBS + """
 m = rw.Mlp(np.zeros(6, np.float32), np.ones(6, np.float32), stream=0)
-base, row, full = lib.fake_plain_bytes(), 5 * 128 * 4, 2 * 152 * 8 * 16
+row, full = 5 * 128 * 4, 2 * 152 * 8 * 16
 held = []
 for n in (10, 7, 1000, 1001, 5, full + 1, 3 * full):
     m.gradient(np.zeros((n, 6), np.float32), np.zeros(n, np.float32), np.array([0, n], np.int32))
-    held.append((lib.fake_plain_bytes() - base) // row)
+    held.append(lib.fake_pool_used() // row)
 assert held == [10, 10, 1000, 1500, 1500, full, full], held
 m.close()
-assert lib.fake_plain_bytes() == 0
+assert lib.fake_plain_bytes() == 0 and lib.fake_pool_used() == 0 and lib.fake_bad_frees() == 0
 """)
 
 
