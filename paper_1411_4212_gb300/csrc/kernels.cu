@@ -391,10 +391,8 @@ __global__ void merge_avg_kernel(const MergeArgs a) {
 // (2) per pair of windows (k, k+1), one warp: the interior overlap bin where the central-difference slopes of
 // the averages differ least (lowest bin on ties) into bstar[k], and the step of the shift there, A_k - A_{k+1},
 // into out[k] (out has at least h bins and is assembled afterwards).
-__global__ void merge_pairs_kernel(const MergeArgs a) {
+__device__ __forceinline__ void merge_pair(const MergeArgs& a, int k) {
   const int lane = threadIdx.x & 31;
-  const int k = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  if (k + 1 >= a.h) return;
   const int W = a.W;
   const int sk = a.starts[k], sn = a.starts[k + 1];
   const int lo = sn + 1, hi = sk + W - 2;
@@ -426,13 +424,23 @@ __global__ void merge_pairs_kernel(const MergeArgs a) {
   }
 }
 
+__global__ void merge_pairs_kernel(const MergeArgs a) {
+  const int k = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  if (k + 1 < a.h) merge_pair(a, k);
+}
+
+// Few pairs, at most one for each warp of the kernel that follows, go along with that kernel: a launch of their own
+// is 2 us of the 43 that joining a small run and reading the curve takes.  But in one SM their FP64 operations take
+// about 2 cycles per bin of every pair, so only up to 1024 bins in all (1 us).
+bool pairs_along(const MergeArgs& a) { return a.h - 1 <= 32 && (long long)(a.h - 1) * a.W <= 1024; }
+
 // (3)-(4) shifts, assembly, mean removal.  One CTA; the assembled curve sits in shared memory when it fits (kSmem).
 // What bounds it: two chains of FP64 additions in the canonical order (62 cycles each): h shifts, and B / 32
 // terms per lane of the mean.  The search for a bin's window, one step after the other before, is a binary
 // search: bin b belongs to the first window k whose join bin lies above b, i.e. the first k whose running
 // maximum of join bins does.  Measured (300 windows, 16384 bins): 321 -> 57 us, the pairs above included.
 template <bool kSmem>
-__global__ void __launch_bounds__(1024) merge_join_kernel(const MergeArgs a) {
+__global__ void __launch_bounds__(1024) merge_join_kernel(const MergeArgs a, const int along) {
   extern __shared__ __align__(16) unsigned char js[];
   const int h = a.h, W = a.W, B = a.B;
   double* shift = reinterpret_cast<double*>(js);
@@ -441,6 +449,10 @@ __global__ void __launch_bounds__(1024) merge_join_kernel(const MergeArgs a) {
   int* start = top + h;
   __shared__ double mean_s;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (along) {
+    if (warp + 1 < h) merge_pair(a, warp);
+    __syncthreads();
+  }
   for (int k = threadIdx.x; k < h; k += blockDim.x) {
     shift[k] = k + 1 < h ? a.out[k] : 0.0;
     start[k] = a.starts[k];
@@ -495,18 +507,19 @@ __global__ void __launch_bounds__(1024) merge_join_kernel(const MergeArgs a) {
 
 cudaError_t launch_merge(const MergeArgs& a, cudaStream_t stream) {
   merge_avg_kernel<<<a.h, 256, sizeof(double) * (size_t)a.m, stream>>>(a);
-  if (a.h > 1) merge_pairs_kernel<<<(a.h + 2) / 4, 128, 0, stream>>>(a);
+  const int along = pairs_along(a) ? 1 : 0;
+  if (!along) merge_pairs_kernel<<<(a.h + 2) / 4, 128, 0, stream>>>(a);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   const size_t js = (sizeof(double) + 2 * sizeof(int)) * (size_t)a.h;
   const size_t with_curve = js + sizeof(double) * (size_t)a.B;
   if (with_curve <= 200 * 1024) {          // up to about 25000 bins
     e = cudaFuncSetAttribute(merge_join_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-    if (e == cudaSuccess) merge_join_kernel<true><<<1, 1024, with_curve, stream>>>(a);
+    if (e == cudaSuccess) merge_join_kernel<true><<<1, 1024, with_curve, stream>>>(a, along);
   } else {
     if (js > 48 * 1024)
       e = cudaFuncSetAttribute(merge_join_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)js);
-    if (e == cudaSuccess) merge_join_kernel<false><<<1, 1024, js, stream>>>(a);
+    if (e == cudaSuccess) merge_join_kernel<false><<<1, 1024, js, stream>>>(a, along);
   }
   return e == cudaSuccess ? cudaGetLastError() : e;
 }
