@@ -546,7 +546,8 @@ __device__ double block_sum(double v, double* red) {
 
 // kCached: at most kThermoKept bins per thread, whose weights stay in registers between the passes.
 // What bounds it: FP64 issue.  Per bin and temperature seven FP64 operations are left (of 46 with the library's
-// exponential in both passes and FP64 maxima).  Measured: 281 temperatures x 16384 bins 451 -> 99 us.
+// exponential in both passes and FP64 maxima).  Measured: 281 temperatures x 16384 bins 451 -> 100 us; one bin
+// more, past what the registers hold, takes 131.
 constexpr int kThermoKept = 16;
 template <bool kCached>
 __global__ void __launch_bounds__(1024) thermo_kernel(const double* __restrict__ lng, const double* __restrict__ E,

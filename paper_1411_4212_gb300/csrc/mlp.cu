@@ -23,8 +23,8 @@
 //
 // Measured on GB300 (51 840 samples, one Adam step): 1.49 -> 0.25 ms in kernels (forward 0.27 -> 0.043, backward
 // with the weight gradients 1.14 -> 0.18) against one CTA of 128 threads per SM with FP32 FMAs; the gradient's
-// error against 64 bits 1.9e-7 -> 1.0e-7, the output's 4e-7 -> 2e-7.  Tensor instructions keep the SM 35-45 % busy
-// (644 TFLOP/s is their peak here); the rest is the elementwise part, which two warps per scheduler overlap only
+// error against 64 bits 1.9e-7 -> 1.0e-7, the output's 4e-7 -> 2e-7.  Tensor instructions keep the SM 32-41 % busy
+// (a loop of nothing else reaches 607 TFLOP/s); the rest is the elementwise part, which two warps per scheduler overlap only
 // partly.  (Elementwise work fused between the tensor instructions of the next columns ran slower: the code then
 // exceeds the instruction cache.)
 //

@@ -14,8 +14,8 @@
 //     H at the resulting state.
 // The owner table may alias sites (hashed): an alias names a move that cannot change the field; the
 // producer sorts such bits out by the distance of the sites.  Two record buffers alternate; named barriers
-// READY(b mod 2) and DONE(b mod 2) order the hand-over, so the producer reads the lattice only after every
-// move of batch b-1 has been written.
+// READY(b mod 2) and DONE(b mod 2) order the hand-over, so the producer reads the lattice for batch b after every
+// move of batch b-2 has been written; what batch b-1 changes is corrected.
 #include "walker_common.cuh"
 
 namespace rewl {
@@ -673,8 +673,8 @@ __device__ __forceinline__ void pipe_walk_slot(const WalkerArgs& a, const int sl
     // instruction waits for the one before).  So a round costs as few dependent steps as possible, and
     // rejected moves cost nothing.  Resolving one move after the other, or blocks of 8 with a restart at
     // every event, took 90-350 cycles per move; now (ms per 10^4 moves, GB300) bcc L = 16, 2 shells,
-    // [E_gs, 0], 64 walkers: 0.69 -> 0.47; bcc L = 8, 3 shells, converging (4000 moves): 1.03 -> 0.49;
-    // 576 walkers of bcc L = 4, 5, 6, converging (4000 moves): 3.1 -> 0.66.
+    // [E_gs, 0], 64 walkers: 0.69 -> 0.46; bcc L = 8, 3 shells, converging (4000 moves): 1.03 -> 0.50;
+    // 576 walkers of bcc L = 4, 5, 6, converging (4000 moves): 3.1 -> 0.67.
     // A round finds the first move that counts, and what it does, with one warp minimum (24 cycles; a
     // vote, a find-first-set and a shuffle take 100): key = lane << 27 | payload, all ones for lanes
     // with nothing to say and for decided moves.  One branch per round tells the rare payloads apart.
@@ -1112,9 +1112,9 @@ __device__ __forceinline__ void pipe_walk_slot(const WalkerArgs& a, const int sl
 
 // One CTA per slot; barrier 0 spans the CTA, 1..4 serve the pair.  Lattice in shared memory,
 // arguments as kernel parameters.  The arena holds the lattice, so at bcc L = 16 one CTA fills an
-// SM's shared memory; the register budget is left open (minimum one block per SM), which measured
-// about 1 % faster on GB300 than the default budget.  (Small lattices fit 4 CTAs per SM by
-// registers at this budget.)
+// SM's shared memory; the register budget is left open (minimum one block per SM): bcc L = 16, 2 shells over its full
+// range 3.86 ms with the 109 registers that it takes, 4.16 with the 79 of the default budget; L = 8, 3 shells
+// converging 8.4 and 9.5 (127, 80).  (Small lattices fit 3 or 4 CTAs per SM by registers at this budget.)
 template <bool kTraj, int NSH>
 __global__ void __launch_bounds__(kWalkerThreads, 1) walker_pipe_kernel(const WalkerArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -1126,8 +1126,8 @@ __global__ void __launch_bounds__(kWalkerThreads, 1) walker_pipe_kernel(const Wa
 // L1) and the per-launch moves and recompute flag as parameters.  On GB300 the bcc L = 32
 // four-shell walker ran 25 % faster this way than with parameter arguments, while the
 // shared-memory walker ran 3 % slower, so each keeps its own form.  Register budget: four blocks
-// per SM (128 registers), the residency that runs 512 walkers in one wave at 2048-entry tables;
-// 4 % faster than the default budget (96 registers).
+// per SM (at most 128 registers), the residency that runs 512 walkers in one wave at 2048-entry tables.  (With four
+// shells the default budget gives 128 as well, 9.97 against 9.96 ms of the full range; 96 with fewer.)
 template <bool kTraj, int NSH>
 __global__ void __launch_bounds__(kWalkerThreads, 4)
     walker_pipe_global_kernel(const WalkerArgs* __restrict__ ap, long long moves, int recompute) {
@@ -1141,9 +1141,9 @@ __global__ void __launch_bounds__(kWalkerThreads, 4)
 // with its own shared-memory arena and barriers (1 + 5w .. 5 + 5w).  A job's lattice sits in the
 // arena or stays in global memory (L2) as its smem_lattice flag says.
 // Register budget: at least two blocks of the largest shape per SM (at most 170 registers per
-// thread).  The tunings the autotuner picks are limited by shared memory, not registers; on GB300
-// the 64-job batch ran 7 % faster at this budget (168 registers, no spills) than at the default
-// (96 registers and a spill) and 3 % faster than with the budget fully open.
+// thread; production spills nothing).  64 runs in a batch, 3 shells, three CTAs of two workers per SM: 30.2 ms with
+// 168 registers, 30.0 with the 136 of the default budget, 33.5 with the 198 of an open one (two CTAs per SM); runs of
+// L = 4, 5, 6 converging 12.3, 12.4 and 12.3.
 template <bool kTraj, int NSH>
 __global__ void __launch_bounds__(kBatchMaxWorkers * kWorkerThreads, 2)
     walker_batch_kernel(const WalkerArgs* __restrict__ jobs, const int2* __restrict__ items, int n_items, int* head,
