@@ -92,9 +92,9 @@ typedef struct {
   int32_t mode;                  /* REWL_MODE_PRODUCTION or REWL_MODE_TRAJECTORY */
   int32_t group_size;            /* lanes per trial move (1,2,4,8,16,32) = summation order of the
                                     local field; 0 = choose from N and z.  Production bcc runs
-                                    with 1 take the warp-specialised walker, which is the fastest
-                                    at every size (on small lattices, where 0 picks a group of 4
-                                    to 16 lanes, 1.3 to 3.7 times); another value is another
+                                    with 1 take the warp-specialised walker, the fastest one
+                                    measured at any size (on small lattices, where 0 picks 4
+                                    to 16 lanes, by 1.3 to 3.7 times); another value is another
                                     walk for the same seed, of the same statistics */
   int64_t exchange_interval;     /* trial moves per walker between replica exchanges (> 0) */
   int64_t max_moves_per_stage;   /* cap for rewl_run_stage (moves per walker); 0 = no cap */
